@@ -12,8 +12,9 @@
 // weights are the FP64 value of the definition rounded once to the storage
 // type: for BF16 storage an FP32 value (exponent argument carried in FP64)
 // rounds to the same bf16 except within a few FP32 ulps of a bf16 rounding
-// midpoint, where the FP64 value is computed; FP32 storage, whose rounding
-// step an FP32 estimate cannot decide, always takes the FP64 value.
+// midpoint, where the FP64 value is computed; for FP32 storage a double-float
+// value (about 2^-40) decides the rounding, except within its error bound of an
+// FP32 rounding midpoint.
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -37,6 +38,7 @@ struct HintGeo {
   double xl, yl, wb, hb, iwb2, ihb2;  // bin centres; 2 / w_b, 2 / h_b
   float xlh, xll, ylh, yll;          // x_l, y_l as double-floats
   float iwh, iwl, ihh, ihl;          // 2 / w_b, 2 / h_b as double-floats
+  float tol;                         // relative error bound of a double-float bin weight
   int nbx, nby, hx, hy, gnx, gny;
   int32_t C, Pm, S, Mm;
   int64_t Nst, mv0, bn0, N;
@@ -483,7 +485,7 @@ __global__ void __launch_bounds__(256) k_dens_level(int NB, int L, const int64_t
 __global__ void k_dens_final(HintGeo G, int nlev, const int64_t *boff, const uint32_t *blist,
                              const double *area, LevelBufs lv, const double *amac,
                              double abin, double cap, double mu, double *Db, double *Cb,
-                             double *phi, float *phif) {
+                             double *phi, float *phif, float *phil) {
   const int NB = G.nbx * G.nby;
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < NB; b += gridDim.x * blockDim.x) {
     int L = 0;
@@ -512,6 +514,7 @@ __global__ void k_dens_final(HintGeo G, int nlev, const int64_t *boff, const uin
     Cb[b] = c;
     phi[b] = ph;
     phif[b] = __double2float_rn(ph);
+    phil[b] = __double2float_rn(ph - (double)__double2float_rn(ph));  // ph - phif
   }
 }
 
@@ -681,6 +684,71 @@ __device__ __forceinline__ dfl df_ratio(float x, float c, float h) {
   return df_norm(dfl{q, __fdiv_rn(__fadd_rn(r, d.lo), h)});
 }
 
+// a b as a double-float.
+__device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  float e = __fmaf_rn(a.hi, b.hi, -p);
+  e = __fmaf_rn(a.hi, b.lo, e);
+  e = __fmaf_rn(a.lo, b.hi, e);
+  return df_norm(dfl{p, e});
+}
+// 2^{-j/32}, j = 0..31, as double-floats.
+struct ExpTable {
+  float2 t[32];
+};
+// e^{-r} for 0 <= r < 60 to about 2^-42, in FP32 operations (table-driven
+// exponential after P. T. P. Tang, ACM TOMS 15, 1989): e^{-r} = 2^{-k/32} e^f with
+// k = rint(32 r / ln 2) and |f| <= ln 2 / 64 + a few ulps; ln 2 / 32 in three
+// parts, the first two of 12 bits, so that their products with k are exact; e^f
+// by its Taylor series, the terms from f^3 on in one FP32 Horner form.
+__device__ __forceinline__ dfl exp_neg_dd(dfl r, const float2 *tab) {
+  const float kf = rintf(__fmul_rn(r.hi, 46.166241308446829f));  // 32 / ln 2
+  const int k = (int)kf;
+  constexpr float kL1 = 0x1.62ep-6f, kL2 = 0x1.0bep-20f, kL3 = 0x1.be8e7ap-32f;
+  dfl f{__fmul_rn(kf, kL1), 0.f};
+  df_add(f, -r.hi);
+  df_add(f, __fmul_rn(kf, kL2));
+  f.lo = __fadd_rn(f.lo, __fmaf_rn(kf, kL3, -r.lo));
+  f = df_norm(f);
+  const float q = __fmul_rn(f.hi, f.hi);
+  const float qe = __fmaf_rn(f.hi, f.hi, -q);
+  float c = __fmaf_rn(f.hi, 1.f / 120.f, 1.f / 24.f);
+  c = __fmaf_rn(f.hi, c, 1.f / 6.f);
+  c = __fmul_rn(__fmul_rn(q, f.hi), c);  // f^3 / 6 + f^4 / 24 + f^5 / 120
+  dfl e = f;                              // e^f - 1
+  df_add(e, __fmul_rn(0.5f, q));
+  e.lo = __fadd_rn(e.lo, __fadd_rn(__fmaf_rn(f.hi, f.lo, __fmul_rn(0.5f, qe)), c));
+  e = df_norm(e);
+  const float2 tj = tab[k & 31];
+  dfl t = df_mul(dfl{tj.x, tj.y}, e);
+  dfl s{tj.x, 0.f};
+  df_add(s, t.hi);
+  s.lo = __fadd_rn(s.lo, __fadd_rn(tj.y, t.lo));
+  const float sc = __uint_as_float((uint32_t)(127 - (k >> 5)) << 23);  // exact scaling
+  s = df_norm(s);
+  return dfl{__fmul_rn(s.hi, sc), __fmul_rn(s.lo, sc)};
+}
+// Whether the normalized double-float v, of relative error at most tol, may
+// round to another FP32 value than the one it stands for: v lies within its
+// error of a rounding midpoint, or is too small or an exact power of two (whose
+// midpoints are not half an ulp away on both sides).
+__device__ __forceinline__ bool near_fp32_tie(dfl v, float tol) {
+  const uint32_t b = __float_as_uint(v.hi) & 0x7fffffffu;
+  if ((b & 0x7fffffu) == 0u || b < (40u << 23) || b >= (250u << 23)) return true;
+  const float half = __uint_as_float((b & 0x7f800000u) - (24u << 23));
+  return !(fabsf(fabsf(v.lo) - half) > tol * fabsf(v.hi));
+}
+constexpr float kExpMax = 60.f;        // largest exponent of exp_neg_dd
+constexpr float kMacroTol = 0x1p-39f;  // a macro weight's error bound at ratio 0 ...
+constexpr float kMacroTolR = 0x1p-42f;  // ... and per unit of its ratio
+// -e^{-r} w and -(e phi) w for FP32 storage, rounded once, from double-floats;
+// *tie: the rounding is not decided and the FP64 value is needed.
+__device__ __forceinline__ float df_weight(dfl e, dfl w, float tol, bool *tie) {
+  const dfl v = df_mul(e, w);
+  *tie = near_fp32_tie(v, tol);
+  return -v.hi;
+}
+
 // Hint part of the rows of cells, macro pins and stars (thread per row): for a
 // hint cell its macro entries (ascending macro), written to the row's hm
 // place, and the weights of its detection-window bins as a dense block of W
@@ -691,21 +759,28 @@ __device__ __forceinline__ dfl df_ratio(float x, float c, float h) {
 // sums of the whole augmented row are the static ones plus the hint entries.
 // The window ratios |x - x_b| / (w_b / 2) = |u - (2 xx + 1)|, u = 2 (x - x_l) /
 // w_b, come from u (double-float, once per cell) as exact double-float
-// differences; macro ratios are double-float quotients.  With BF16 storage FP64
-// only recomputes weights near a bf16 rounding midpoint; with FP32 storage
-// every weight is the FP64 value of the definition rounded once.
-constexpr int kAsmStage = 768;  // own entries of a warp's 32 rows staged in shared memory
+// differences; macro ratios are double-float quotients.  FP64 only recomputes
+// weights near a rounding midpoint of the storage type.  For FP32 storage the
+// weight itself is a double-float (exponential to 2^-42, products to 2^-45): its
+// FP64 form, at 1/64 of the FP32 rate, took 352 us of a 210k-cell design's refinement
+// round of 970 us (order 8); with the double-float form the round takes 641 us.
+constexpr int kAsmStage = 752;  // own entries of a warp's 32 rows staged in shared memory
+template <bool bf>
 __global__ void __launch_bounds__(256, 3) k_assemble_hints(
-    HintGeo G, int wdtype, const uint32_t *hrp, const int32_t *longidx, const uint64_t *lptr,
+    HintGeo G, ExpTable xt, const uint32_t *hrp, const int32_t *longidx, const uint64_t *lptr,
     const dfl *sdsum, const dfl *spsum, const uint8_t *hflag, const int32_t *cell_bin,
     const int32_t *n_ovl, const float2 *xy, const float *cw, const float *ch,
     const int64_t *gptr, const uint32_t *glist, const float4 *ggeo, const double *base_w,
-    const float *phif, const double *phid, int W, const int32_t *cmem, const float4 *mgeo,
+    const float *phif, const float *phil, const double *phid, int W, const int32_t *cmem, const float4 *mgeo,
     int32_t *col, void *w, void *bwin, int32_t *hbin, dfl *dsum, dfl *psum, uint64_t *mac_base,
     unsigned long long *counts) {
   __shared__ int32_t stage_col[8][kAsmStage];
   __shared__ uint32_t stage_w[8][kAsmStage];
-  const bool bf = wdtype == PL_W_BF16;
+  __shared__ float2 exp_tab[bf ? 1 : 32];
+  if (!bf) {
+    if (threadIdx.x < 32) exp_tab[threadIdx.x] = xt.t[threadIdx.x];
+    __syncthreads();
+  }
   const int lane = threadIdx.x & 31;
   int32_t *scol = stage_col[threadIdx.x >> 5];
   uint32_t *sw = stage_w[threadIdx.x >> 5];
@@ -755,6 +830,7 @@ __global__ void __launch_bounds__(256, 3) k_assemble_hints(
       };
       if (!isfinite(p.x) || !isfinite(p.y)) p = make_float2(0.f, 0.f);
       const float bwf = __double2float_rn(bw);
+      const dfl bwd{bwf, bf ? 0.f : __double2float_rn(bw - (double)bwf)};
       // macro entries, ascending macro id (grid bucket lists are sorted)
       uint64_t k = mb;
       auto mac_entry = [&](int m, float4 mg) {
@@ -770,7 +846,13 @@ __global__ void __launch_bounds__(256, 3) k_assemble_hints(
           bits = h;
           sv = bf16_to_f(h);
         } else {
-          sv = __double2float_rn(macro_w_exact(p.x, p.y, mg.x, mg.y, mg.z, mg.w, bw));
+          const dfl rx = df_ratio(p.x, mg.x, __fmul_rn(0.5f, mg.z));
+          const dfl ry = df_ratio(p.y, mg.y, __fmul_rn(0.5f, mg.w));
+          const dfl r = df_ge(rx, ry) ? rx : ry;
+          bool tie = !(r.hi < kExpMax);
+          sv = 0.f;
+          if (!tie) sv = df_weight(exp_neg_dd(r, exp_tab), bwd, kMacroTol + kMacroTolR * r.hi, &tie);
+          if (tie) sv = __double2float_rn(macro_w_exact(p.x, p.y, mg.x, mg.y, mg.z, mg.w, bw));
           bits = __float_as_uint(sv);
         }
         put(k, (int32_t)(G.mv0 + m), bits);
@@ -845,46 +927,79 @@ __global__ void __launch_bounds__(256, 3) k_assemble_hints(
             wb16[sidx++] = h;
           }
         }
-      } else
-      for (int yy = by - G.hy; yy <= by + G.hy; ++yy) {
-        const bool yin = yy >= 0 && yy < G.nby;
-        // e^{-max(rx, ry)} is e^{-rx} or e^{-ry}
-        const dfl ry = df_absdiff(uy.hi, uy.lo, (float)(2 * yy + 1));
-        const float ey = (bf && yin) ? exp_neg_df(ry) : 0.f;
-        for (int xc = bx - G.hx; xc <= bx + G.hx; xc += 4) {
-          float ph[4];  // four window bins' phi loaded at once
+      } else if (bf) {
+        for (int yy = by - G.hy; yy <= by + G.hy; ++yy) {
+          const bool yin = yy >= 0 && yy < G.nby;
+          // e^{-max(rx, ry)} is e^{-rx} or e^{-ry}
+          const dfl ry = df_absdiff(uy.hi, uy.lo, (float)(2 * yy + 1));
+          const float ey = yin ? exp_neg_df(ry) : 0.f;
+          for (int xc = bx - G.hx; xc <= bx + G.hx; xc += 4) {
+            float ph[4];  // four window bins' phi loaded at once
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int xx = xc + u;
-            ph[u] = (yin && xx >= 0 && xx < G.nbx && xx <= bx + G.hx) ? phif[yy * G.nbx + xx] : 0.f;
-          }
+            for (int u = 0; u < 4; ++u) {
+              const int xx = xc + u;
+              ph[u] = (yin && xx >= 0 && xx < G.nbx && xx <= bx + G.hx) ? phif[yy * G.nbx + xx] : 0.f;
+            }
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int xx = xc + u;
-            if (xx > bx + G.hx) break;
-            uint32_t bits = 0;
-            if (yin && xx >= 0 && xx < G.nbx) {
-              const int bb = yy * G.nbx + xx;
-              float sv;
-              if (bf) {
+            for (int u = 0; u < 4; ++u) {
+              const int xx = xc + u;
+              if (xx > bx + G.hx) break;
+              uint16_t h = 0;
+              if (yin && xx >= 0 && xx < G.nbx) {
                 const dfl rx = df_absdiff(ux.hi, ux.lo, (float)(2 * xx + 1));
                 const float e = df_ge(rx, ry) ? exp_neg_df(rx) : ey;
                 const float wv = -((e * ph[u]) * bwf);
-                const uint16_t h = near_bf16_tie(wv)
-                                       ? d2bf16(bin_w_exact(p.x, p.y, xx, yy, G, phid[bb], bw))
-                                       : f2bf16(wv);
-                bits = h;
-                sv = bf16_to_f(h);
-              } else {
-                sv = __double2float_rn(bin_w_exact(p.x, p.y, xx, yy, G, phid[bb], bw));
-                bits = __float_as_uint(sv);
+                h = near_bf16_tie(wv)
+                        ? d2bf16(bin_w_exact(p.x, p.y, xx, yy, G, phid[yy * G.nbx + xx], bw))
+                        : f2bf16(wv);
+                acc_deg(Dl, Pl, bf16_to_f(h));
+                ++slots;
               }
-              acc_deg(Dl, Pl, sv);
-              ++slots;
+              wb16[sidx++] = h;
             }
-            if (bf) wb16[sidx] = (uint16_t)bits;
-            else wb32[sidx] = bits;
-            ++sidx;
+          }
+        }
+      } else {
+        // FP32 storage: double-float weights; the ratios and exponentials of
+        // three window columns once per cell (wider windows: per slot)
+        const bool three = G.hx == 1;
+        dfl rxs[3], exs[3];
+        auto column = [&](int xx, dfl *r, dfl *e) {
+          *r = df_absdiff(ux.hi, ux.lo, (float)(2 * xx + 1));
+          *e = r->hi < kExpMax ? exp_neg_dd(*r, exp_tab) : dfl{0.f, 0.f};
+        };
+        if (three) {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) column(bx - 1 + c, &rxs[c], &exs[c]);
+        }
+        auto slot = [&](int xx, int yy, bool yin, dfl rx, dfl ex, dfl ry, dfl ey) {
+          float sv = 0.f;
+          if (yin && xx >= 0 && xx < G.nbx) {
+            const int bb = yy * G.nbx + xx;
+            const bool ge = df_ge(rx, ry);
+            const dfl e = df_mul(ge ? ex : ey, dfl{phif[bb], phil[bb]});
+            bool tie;
+            sv = df_weight(e, bwd, G.tol, &tie);
+            if (tie || !((ge ? rx.hi : ry.hi) < kExpMax))
+              sv = __double2float_rn(bin_w_exact(p.x, p.y, xx, yy, G, phid[bb], bw));
+            acc_deg(Dl, Pl, sv);
+            ++slots;
+          }
+          wb32[sidx++] = __float_as_uint(sv);
+        };
+        for (int yy = by - G.hy; yy <= by + G.hy; ++yy) {
+          const bool yin = yy >= 0 && yy < G.nby;
+          const dfl ry = df_absdiff(uy.hi, uy.lo, (float)(2 * yy + 1));
+          const dfl ey = ry.hi < kExpMax ? exp_neg_dd(ry, exp_tab) : dfl{0.f, 0.f};
+          if (three) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) slot(bx - 1 + c, yy, yin, rxs[c], exs[c], ry, ey);
+          } else {
+            for (int xx = bx - G.hx; xx <= bx + G.hx; ++xx) {
+              dfl rx, ex;
+              column(xx, &rx, &ex);
+              slot(xx, yy, yin, rx, ex, ry, ey);
+            }
           }
         }
       }
@@ -1102,6 +1217,13 @@ static HintGeo make_geo(const pl_graph *g) {
   split(G.yl, &G.ylh, &G.yll);
   split(G.iwb2, &G.iwh, &G.iwl);
   split(G.ihb2, &G.ihh, &G.ihl);
+  // Error bound of a double-float bin weight against the FP64 one, relative:
+  // the exponential and the products (2^-41), the ratio 2 (x - x_l) / w_b (its
+  // double-float form carries about 2^-45 of the bin count and 2^-47 of the
+  // region's coordinates over the bin size; the FP64 form far less).
+  G.tol = (float)(std::ldexp(1.0, -39) + std::ldexp((double)g->nbx + g->nby, -43) +
+                  std::ldexp(std::fmax(std::fabs(g->xl), std::fabs(g->xh)) / g->wb +
+                                 std::fmax(std::fabs(g->yl), std::fabs(g->yh)) / g->hb, -44));
   G.nbx = g->nbx;
   G.nby = g->nby;
   G.hx = g->hx;
@@ -1117,6 +1239,19 @@ static HintGeo make_geo(const pl_graph *g) {
   G.bn0 = g->Nst + g->Mm;
   G.N = g->N;
   return G;
+}
+
+static const ExpTable &exp_table() {
+  static const ExpTable t = [] {
+    ExpTable e;
+    for (int j = 0; j < 32; ++j) {
+      const double v = std::exp2(-(double)j / 32.0);
+      e.t[j].x = (float)v;
+      e.t[j].y = (float)(v - (double)e.t[j].x);
+    }
+    return e;
+  }();
+  return t;
 }
 
 static BinGeo make_bingeo(const pl_graph *g) {
@@ -1387,8 +1522,8 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   cudaStream_t s2 = g->side, s3 = g->side2;
   TRY(ensure(g->Db, (size_t)NB * 8 + 16));
   TRY(ensure(g->phi, (size_t)NB * 8 + 16));
-  TRY(ensure(g->tmp[4], (size_t)NB * 4 + 256));
-  float *phif = P<float>(g->tmp[4]);
+  TRY(ensure(g->tmp[4], (size_t)NB * 8 + 256));
+  float *phif = P<float>(g->tmp[4]), *phil = phif + NB;  // phi_b as double-floats
   TRY(cudaEventRecord(g->ev_fork, s));
   TRY(cudaStreamWaitEvent(s2, g->ev_fork, 0));
   TRY(cudaStreamWaitEvent(s3, g->ev_fork, 0));
@@ -1436,7 +1571,7 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   k_dens_final<<<grid_for(NB, 32), 32, 0, s2>>>(  // a warp per 32 bins: spread over the SMs
       G, nlev, P<int64_t>(g->boff), P<uint32_t>(g->blist), P<double>(g->carea), lv,
       P<double>(g->amac), g->abin, p->capacity, p->mu, P<double>(g->Db), P<double>(g->Cb),
-      P<double>(g->phi), phif);
+      P<double>(g->phi), phif, phil);
   note_launch();
   TRY(cudaEventRecord(g->ev_join, s2));
   TRY(cudaEventRecord(g->ev_join2, s3));
@@ -1463,11 +1598,12 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   TRY(cudaMemsetAsync(counts, 0, 16, s));
   TRY(cudaStreamWaitEvent(s, g->ev_join, 0));   // phi
   TRY(cudaStreamWaitEvent(s, g->ev_join2, 0));  // the macro lists
-  k_assemble_hints<<<grid_for(g->Nst, 256), 256, 0, s>>>(
-      G, g->wdtype, P<uint32_t>(m.rp_s), P<int32_t>(m.longidx), P<uint64_t>(m.lptr),
+  (g->wdtype == PL_W_BF16 ? k_assemble_hints<true> : k_assemble_hints<false>)
+      <<<grid_for(g->Nst, 256), 256, 0, s>>>(
+      G, exp_table(), P<uint32_t>(m.rp_s), P<int32_t>(m.longidx), P<uint64_t>(m.lptr),
       P<dfl>(g->st.dsum), P<dfl>(g->st.psum), P<uint8_t>(g->hflag), P<int32_t>(g->cell_bin),
       P<int32_t>(g->n_ovl), xy, P<float>(g->cw), P<float>(g->ch), P<int64_t>(g->gptr),
-      P<uint32_t>(g->glist), P<float4>(g->ggeo), P<double>(g->base_w), phif, P<double>(g->phi),
+      P<uint32_t>(g->glist), P<float4>(g->ggeo), P<double>(g->base_w), phif, phil, P<double>(g->phi),
       W, cmem_ok ? P<int32_t>(g->cmem) : nullptr, P<float4>(g->mgeo), P<int32_t>(m.col), m.w.p,
       g->hbw.p, P<int32_t>(g->hbin), P<dfl>(m.dsum), P<dfl>(m.psum), P<uint64_t>(g->mac_base),
       counts);

@@ -151,7 +151,7 @@ double workspace_bound(const pl_netlist *nl, const pl_params *p) {
   h.add(seg_b(Mm, nml));
   h.add(NB * 8 + 16);
   h.add(NB * 8 + 16);
-  h.add(NB * 4 + 256);
+  h.add(NB * 8 + 256);
   {
     double tot = 0.0, prev = nmov;
     for (int k = 0; k < 8; ++k) {
