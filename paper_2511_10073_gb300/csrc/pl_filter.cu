@@ -1355,8 +1355,12 @@ __device__ __forceinline__ void batch_units(const StepArgs *As, const long long 
     } else if (K == BK_HUB) {
       warp_chunk<WT, MODE>(A, (int)k);
     } else {
-      if (k < A.bchunk[A.B.NB])
-        bin_chunk<WT, false>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, k);
+      if (k < A.bchunk[A.B.NB]) {
+        if (A.B.W == 9)
+          bin_chunk<WT, false, true>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, k);
+        else
+          bin_chunk<WT, false, false>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, k);
+      }
     }
   }
 }

@@ -1032,7 +1032,8 @@ __global__ void __launch_bounds__(256, 3) k_assemble_hints(
 // position boff[2b] + (c - bchunk[b]) kBinChunk + i of its bin b) goes to
 // out[(c W + t) kBinChunk + i], so the bin rows read each slot of a chunk as
 // consecutive weights.  A thread per (chunk, cell) gathers the cell's block
-// and writes its W weights; places past a bucket's last hint cell get 0.
+// and writes its W weights; places past a bucket's last hint cell are not
+// written (and never read).
 template <typename T>
 __global__ void k_blocks_to_chunks(long long nthreads, int W, const int32_t *bchunk, int NB,
                                    const int32_t *cown, const int64_t *boff,
@@ -1048,8 +1049,6 @@ __global__ void k_blocks_to_chunks(long long nthreads, int W, const int32_t *bch
     if (k < boff[2 * b + 1]) {
       const T *src = blk + (size_t)blist[k] * W;
       for (int t = 0; t < W; ++t) dst[(size_t)t * kBinChunk] = src[t];
-    } else {
-      for (int t = 0; t < W; ++t) dst[(size_t)t * kBinChunk] = (T)0;
     }
   }
 }
