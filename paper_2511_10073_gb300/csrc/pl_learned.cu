@@ -61,14 +61,15 @@ constexpr int SM_W1 = 20480;     // B of layer 1: 64 x 16 BF16
 constexpr int SM_W2 = 22528;     // B of layer 2: 16 x 64 BF16 (four 512 B slabs)
 constexpr int SM_B1 = 24576;     // float [64]
 constexpr int SM_PRM = 24832;    // float mu[16], isd[16], theta[4], b2[4]
-constexpr int SM_W2F = 25088;    // float [4][64]: W2 as BF16 values (backward)
+constexpr int SM_W2F = 25088;    // float [64][4]: W2 as BF16 values, a hidden unit's four together (backward)
 constexpr int SM_BAR = 26112;    // mbarrier
 constexpr int SM_TMEM = 26120;   // tensor memory base address
 constexpr int SM_TC = 26240;     // end of the forward's part
-// training's part (floats, padded strides)
-constexpr int kDhS = kHid + 1, kXsS = kNF + 1;
-constexpr int SM_DH = SM_TC;                        // [128][65]
-constexpr int SM_XS = SM_DH + kTile * kDhS * 4;      // [128][17]
+// training's part (floats; row strides that keep 16- and 8-byte reads aligned
+// and spread the rows' 16-byte stores over the banks)
+constexpr int kDhS = kHid + 4, kXsS = kNF + 2;
+constexpr int SM_DH = SM_TC;                        // [128][68]
+constexpr int SM_XS = SM_DH + kTile * kDhS * 4;      // [128][18]
 constexpr int SM_DO = SM_XS + kTile * kXsS * 4;      // [128][4]
 constexpr int SM_GT = SM_DO + kTile * 4 * 4;         // [128][4]: theta terms, loss
 constexpr int SM_TR = SM_GT + kTile * 4 * 4;
@@ -190,7 +191,7 @@ __device__ uint32_t tc_setup(uint8_t *sm, const float *w) {
     const int n = i / kHid, j = i % kHid;
     const uint16_t b = n < kNOut ? f2bf16(w[kW2 + n * kHid + j]) : (uint16_t)0;
     *reinterpret_cast<uint16_t *>(sm + SM_W2 + opnd_off(n, j, 512)) = b;
-    if (n < kNOut) w2f[n * kHid + j] = bf16_to_f(b);
+    if (n < kNOut) w2f[j * kNOut + n] = bf16_to_f(b);
   }
   float *b1 = reinterpret_cast<float *>(sm + SM_B1);
   float *prm = reinterpret_cast<float *>(sm + SM_PRM);
@@ -589,8 +590,6 @@ __global__ void __launch_bounds__(kTile) k_train_tile(const float *rec, int64_t 
                                                       float inv_n, const float *w, float *part,
                                                       int *status) {
   uint8_t *sm = smem_base();
-  const uint32_t tmem = tc_setup(sm, w);
-  const float *prm = reinterpret_cast<const float *>(sm + SM_PRM);
   const int t = threadIdx.x;
   const int64_t tile = tiles ? (int64_t)tiles[blockIdx.x] : tile0 + blockIdx.x;
   const int64_t i = tile * kTile + t;
@@ -603,6 +602,9 @@ __global__ void __launch_bounds__(kTile) k_train_tile(const float *rec, int64_t 
     for (int k = 0; k < kNF; ++k) q.f[k] = 0.f;
     q.G[0][0] = q.G[0][1] = q.G[1][0] = q.G[1][1] = q.G[2][0] = q.G[2][1] = q.T[0] = q.T[1] = 0.f;
   }
+  // the record's loads are in flight during the setup
+  const uint32_t tmem = tc_setup(sm, w);
+  const float *prm = reinterpret_cast<const float *>(sm + SM_PRM);
   uint32_t xw[8];
   normalise(sm, q.f, xw);
   float o[kNOut];
@@ -639,78 +641,148 @@ __global__ void __launch_bounds__(kTile) k_train_tile(const float *rec, int64_t 
   d[1] = dP[0] * (q.G[2][0] - q.G[0][0]) + dP[1] * (q.G[2][1] - q.G[0][1]);
   d[2] = dP[0];
   d[3] = dP[1];
+  *reinterpret_cast<float4 *>(dout + t * 4) = make_float4(d[0], d[1], d[2], d[3]);
+  *reinterpret_cast<float4 *>(gth + t * 4) =
+      make_float4(dP[0] * q.G[0][0] + dP[1] * q.G[0][1], dP[0] * q.G[1][0] + dP[1] * q.G[1][1],
+                  dP[0] * q.G[2][0] + dP[1] * q.G[2][1], l * inv_n);
 #pragma unroll
-  for (int m = 0; m < kNOut; ++m) dout[t * 4 + m] = d[m];
-  gth[t * 4 + 0] = dP[0] * q.G[0][0] + dP[1] * q.G[0][1];
-  gth[t * 4 + 1] = dP[0] * q.G[1][0] + dP[1] * q.G[1][1];
-  gth[t * 4 + 2] = dP[0] * q.G[2][0] + dP[1] * q.G[2][1];
-  gth[t * 4 + 3] = l * inv_n;
+  for (int j = 0; j < kHid; j += 4) {
+    float h[4];
 #pragma unroll
-  for (int j = 0; j < kHid; ++j) {
-    float s = d[0] * w2f[j];
-    s += d[1] * w2f[kHid + j];
-    s += d[2] * w2f[2 * kHid + j];
-    s += d[3] * w2f[3 * kHid + j];
-    dh[t * kDhS + j] = (pos >> j) & 1u ? s : 0.f;
-  }
-#pragma unroll
-  for (int k = 0; k < kNF; k += 2) {
-    xs[t * kXsS + k] = bf16_to_f((uint16_t)(xw[k / 2] & 0xffffu));
-    xs[t * kXsS + k + 1] = bf16_to_f((uint16_t)(xw[k / 2] >> 16));
-  }
-  __syncthreads();
-  float *row = part + (int64_t)blockIdx.x * kPart;
-  constexpr int nout = kHid * kNF + kHid + kNOut * kHid + kNOut + 3 + 1;
-  for (int oi = t; oi < nout; oi += kTile) {
-    float s = 0.f;
-    int dst;
-    if (oi < kHid * kNF) {
-      const int j = oi / kNF, k = oi % kNF;
-      for (int r = 0; r < kTile; ++r) s += dh[r * kDhS + j] * xs[r * kXsS + k];
-      dst = kW1 + oi;
-    } else if (oi < kHid * kNF + kHid) {
-      const int j = oi - kHid * kNF;
-      for (int r = 0; r < kTile; ++r) s += dh[r * kDhS + j];
-      dst = kB1 + j;
-    } else if (oi < kHid * kNF + kHid + kNOut * kHid) {
-      const int u = oi - kHid * kNF - kHid, m = u / kHid, j = u % kHid;
-      for (int r = 0; r < kTile; ++r)
-        s += dout[r * 4 + m] * bf16_to_f(*reinterpret_cast<const uint16_t *>(sm + SM_HA + opnd_off(r, j, 4096)));
-      dst = kW2 + u;
-    } else if (oi < kHid * kNF + kHid + kNOut * kHid + kNOut) {
-      const int m = oi - (kHid * kNF + kHid + kNOut * kHid);
-      for (int r = 0; r < kTile; ++r) s += dout[r * 4 + m];
-      dst = kB2 + m;
-    } else {
-      const int m = oi - (kHid * kNF + kHid + kNOut * kHid + kNOut);  // 0..2 theta, 3 loss
-      for (int r = 0; r < kTile; ++r) s += gth[r * 4 + m];
-      dst = m < 3 ? kTH + m : kLW;
+    for (int u = 0; u < 4; ++u) {
+      const float4 wj = *reinterpret_cast<const float4 *>(w2f + (j + u) * kNOut);
+      float v = d[0] * wj.x;
+      v += d[1] * wj.y;
+      v += d[2] * wj.z;
+      v += d[3] * wj.w;
+      h[u] = (pos >> (j + u)) & 1u ? v : 0.f;
     }
-    row[dst] = s;
+    *reinterpret_cast<float4 *>(dh + t * kDhS + j) = make_float4(h[0], h[1], h[2], h[3]);
+  }
+#pragma unroll
+  for (int k = 0; k < kNF; k += 2)
+    *reinterpret_cast<float2 *>(xs + t * kXsS + k) = make_float2(
+        bf16_to_f((uint16_t)(xw[k / 2] & 0xffffu)), bf16_to_f((uint16_t)(xw[k / 2] >> 16)));
+  __syncthreads();
+  // The tile's gradient sums, each over the records in order.  A thread forms
+  // a 4 x 2 block of W1's (16 x 8 blocks of 4 hidden units x 2 inputs: two
+  // shared-memory reads per record for eight FMAs; one sum at a time took two
+  // reads per FMA) and b1's sums of its units, then two of W2's, and eight
+  // threads the rest.
+  float *row = part + (int64_t)blockIdx.x * kPart;
+  {
+    const int j0 = (t >> 3) * 4, k0 = (t & 7) * 2;
+    float g[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, gb[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+    for (int r = 0; r < kTile; ++r) {
+      const float4 h = *reinterpret_cast<const float4 *>(dh + r * kDhS + j0);
+      const float2 x = *reinterpret_cast<const float2 *>(xs + r * kXsS + k0);
+      const float hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        g[u][0] += hv[u] * x.x;
+        g[u][1] += hv[u] * x.y;
+        gb[u] += hv[u];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      row[kW1 + (j0 + u) * kNF + k0] = g[u][0];
+      row[kW1 + (j0 + u) * kNF + k0 + 1] = g[u][1];
+      if (k0 == 0) row[kB1 + j0 + u] = gb[u];
+    }
+  }
+  {
+    // output m, hidden units j and j + 1 (a warp's 16 units lie in one slab, so
+    // its reads meet at most two rows of a bank)
+    const int m = t & 3, j = (t >> 2) * 2;
+    float g0 = 0.f, g1 = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < kTile; ++r) {
+      const uint32_t h = *reinterpret_cast<const uint32_t *>(sm + SM_HA + opnd_off(r, j, 4096));
+      const float e = dout[r * 4 + m];
+      g0 += e * __uint_as_float(h << 16);
+      g1 += e * __uint_as_float(h & 0xffff0000u);
+    }
+    row[kW2 + m * kHid + j] = g0;
+    row[kW2 + m * kHid + j + 1] = g1;
+  }
+  if (t < 8) {  // b2, then theta and the loss
+    const float *src = t < 4 ? dout + t : gth + (t - 4);
+    float v = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < kTile; ++r) v += src[r * 4];
+    row[t < 4 ? kB2 + t : t < 7 ? kTH + (t - 4) : kLW] = v;
   }
   tc_teardown(tmem);
 }
 
-// acc[i] (+)= sum over blocks b (in order) of part[b][i], for the trained
-// weights and the loss (i >= kTH).
-__global__ void k_reduce_parts(const float *part, int nblk, double *acc, int first) {
-  const int i = kTH + blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= kPart) return;
-  double s = first ? 0.0 : acc[i];
-  for (int b = 0; b < nblk; ++b) s += (double)part[(int64_t)b * kPart + i];
-  acc[i] = s;
+// A float as a double by integer operations (a conversion takes the FP64 pipe,
+// 1/64 of the FP32 rate); values whose double needs more than a rebased
+// exponent (zero, subnormal, infinite, NaN) are converted.
+__device__ __forceinline__ double f2d(float f) {
+  const uint32_t b = __float_as_uint(f), e = (b >> 23) & 0xffu;
+  if (e - 1u >= 254u) return (double)f;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))),
+                          (int)(b << 29));
 }
 
-// One Adam step on every trained weight from the summed gradient; the
+// FP64 sum over blocks b of part[b][i] for weight i = kTH + 32 blockIdx.x + lane:
+// eight runs of consecutive blocks, a warp each (sixteen loads in flight), every
+// run in block order, then the runs in order.  Returned to warp 0.  A dependent
+// FP64 addition takes about 60 ns here, so one chain over a step's 128 blocks is
+// the whole cost: the sum and its Adam update took 16.2 us a step as a chain per
+// weight (and two launches), 13.4 us with the loads taken off the chain, 5.8
+// us as eight chains.
+constexpr int kSegs = 8;
+__device__ __forceinline__ double sum_parts(const float *part, int nblk, double (*sh)[32]) {
+  const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+  const int i = kTH + blockIdx.x * 32 + lane;
+  const int per = (nblk + kSegs - 1) / kSegs, b1 = min(nblk, (seg + 1) * per);
+  double s = 0.0;
+  for (int b = seg * per; b < b1; b += 16) {
+    float v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v[u] = b + u < b1 && i < kPart ? part[(int64_t)(b + u) * kPart + i] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) s += f2d(v[u]);
+  }
+  sh[seg][lane] = s;
+  __syncthreads();
+  if (seg) return 0.0;
+#pragma unroll
+  for (int k = 1; k < kSegs; ++k) s += sh[k][lane];
+  return s;
+}
+constexpr int kPartGrid = (kPart - kTH + 31) / 32;
+
+// acc[i] (+)= the blocks' sum, for the trained weights and the loss (i >= kTH).
+__global__ void __launch_bounds__(32 * kSegs) k_reduce_parts(const float *part, int nblk,
+                                                             double *acc, int first) {
+  __shared__ double sh[kSegs][32];
+  const int i = kTH + blockIdx.x * 32 + threadIdx.x;
+  const bool mine = threadIdx.x < 32 && i < kPart;
+  const double s = sum_parts(part, nblk, sh);
+  if (mine) acc[i] = first ? s : acc[i] + s;
+}
+
+// One Adam step on every trained weight from the blocks' summed gradient; the
 // minibatch loss is added to *loss.
-__global__ void k_adam(const double *acc, float *w, float *m, float *v, float lr, float b1,
-                       float b2, float eps, float bc1, float bc2, double *loss) {
-  const int i = kTH + blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == kLW) *loss += acc[kLW];
-  if (i >= kLW) return;
-  const float g = (float)acc[i];
-  const float mi = b1 * m[i] + (1.f - b1) * g;
-  const float vi = b2 * v[i] + (1.f - b2) * g * g;
+__global__ void __launch_bounds__(32 * kSegs) k_adam(const float *part, int nblk, float *w, float *m,
+                                                     float *v, float lr, float b1, float b2,
+                                                     float eps, float bc1, float bc2, double *loss) {
+  __shared__ double sh[kSegs][32];
+  const double s = sum_parts(part, nblk, sh);
+  const int i = kTH + blockIdx.x * 32 + threadIdx.x;
+  if (threadIdx.x >= 32 || i > kLW) return;
+  if (i == kLW) {
+    *loss += s;
+    return;
+  }
+  const float g = (float)s;
+  // (roundings written out, so that no change of the code around them moves them)
+  const float mi = __fmaf_rn(b1, m[i], __fmul_rn(1.f - b1, g));
+  const float vi = __fmaf_rn(b2, v[i], __fmul_rn(__fmul_rn(1.f - b2, g), g));
   m[i] = mi;
   v[i] = vi;
   w[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
@@ -721,25 +793,65 @@ __global__ void k_acc_to_grad(const double *acc, float *grad) {
   if (i < kLW) grad[i] = i < kTH ? 0.f : (float)acc[i];
 }
 
+// Reduce-scatter of the N doubles v over the warp: on return the lane with
+// cnt = 1 holds the warp's sum of value pos in v[0] (as warp_rs_df).
+template <int N, int M>
+__device__ __forceinline__ void warp_rs_d(double *v, int &pos, int &cnt) {
+  constexpr int H = (N + 1) / 2;
+  const bool hi = (threadIdx.x & M) != 0;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const double a = v[i], b = i + H < N ? v[i + H] : 0.0;
+    v[i] = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, M);
+  }
+  if (hi) {
+    pos += H;
+    cnt = cnt > H ? cnt - H : 0;
+  } else {
+    cnt = cnt < H ? cnt : H;
+  }
+  if constexpr (M > 1) warp_rs_d<H, M / 2>(v, pos, cnt);
+}
+
 // Per-block FP64 sums over records: sum f_k, sum f_k^2, and the normal
 // equations of the taps (A = sum G G^T over both axes, 6 entries; b = sum G T).
-__global__ void k_rec_stats(const float *rec, int64_t nrec, double *part) {
+// FP64 bound: conversions are integer operations, a feature that is zero in
+// the whole warp (unused features, flags) adds nothing and is skipped, and the
+// threads' sums meet by halves of the block (warps 4..7 to 0..3, 2..3 to 0..1,
+// 1 to 0, then a reduce-scatter over the lanes): one tree for all 41 sums, the
+// same tree as a sum over a shared array of 256, whose nine barriers per sum it
+// replaces.  630k records: 270 -> 109 us, and their final sum 63 -> 39 us.
+// (The blocks, the trees and the order of the final sums are part of the result:
+// the taps' normal equations are nearly singular where the taps are close to
+// one another, and the solution shows the sums' last bits.)
+__global__ void __launch_bounds__(256) k_rec_stats(const float *rec, int64_t nrec, double *part) {
+  __shared__ double sh[kStats][128];
   double s[kStats];
 #pragma unroll
   for (int k = 0; k < kStats; ++k) s[k] = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nrec;
-       i += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); i0 < nrec; i0 += stride) {
+    const int64_t i = i0 + (threadIdx.x & 31);
     RecIn q;
-    load_rec(rec, i, q);
+    if (i < nrec) {
+      load_rec(rec, i, q);
+    } else {
+#pragma unroll
+      for (int k = 0; k < kNF; ++k) q.f[k] = 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) q.G[k][0] = q.G[k][1] = 0.f;
+      q.T[0] = q.T[1] = 0.f;
+    }
 #pragma unroll
     for (int k = 0; k < kNF; ++k) {
-      const double f = q.f[k];
+      if (!__any_sync(0xffffffffu, q.f[k] != 0.f)) continue;  // (NaN is not 0)
+      const double f = f2d(q.f[k]);
       s[k] += f;
       s[16 + k] += f * f;
     }
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const double a = q.G[0][c], b = q.G[1][c], d = q.G[2][c], T = q.T[c];
+      const double a = f2d(q.G[0][c]), b = f2d(q.G[1][c]), d = f2d(q.G[2][c]), T = f2d(q.T[c]);
       s[32] += a * a;
       s[33] += a * b;
       s[34] += a * d;
@@ -751,25 +863,39 @@ __global__ void k_rec_stats(const float *rec, int64_t nrec, double *part) {
       s[40] += d * T;
     }
   }
-  __shared__ double sh[256];
 #pragma unroll
-  for (int k = 0; k < kStats; ++k) {
-    sh[threadIdx.x] = s[k];
-    __syncthreads();
-    for (int d = 128; d > 0; d >>= 1) {
-      if (threadIdx.x < d) sh[threadIdx.x] += sh[threadIdx.x + d];
-      __syncthreads();
+  for (int d = 128; d >= 32; d >>= 1) {
+    if ((int)threadIdx.x >= d && (int)threadIdx.x < 2 * d) {
+#pragma unroll
+      for (int k = 0; k < kStats; ++k) sh[k][threadIdx.x - d] = s[k];
     }
-    if (threadIdx.x == 0) part[(int64_t)blockIdx.x * kStats + k] = sh[0];
+    __syncthreads();
+    if ((int)threadIdx.x < d) {
+#pragma unroll
+      for (int k = 0; k < kStats; ++k) s[k] += sh[k][threadIdx.x];
+    }
     __syncthreads();
   }
+  if (threadIdx.x >= 32) return;
+  int pos = 0, cnt = kStats;
+  warp_rs_d<kStats, 16>(s, pos, cnt);
+  // (41 values over 32 lanes: a lane is left with one or two)
+  double *dst = part + (int64_t)blockIdx.x * kStats;
+  if (cnt > 0) dst[pos] = s[0];
+  if (cnt > 1) dst[pos + 1] = s[1];
 }
 
-__global__ void k_stats_final(const double *part, int nblk, double *out) {
-  const int k = threadIdx.x;
-  if (k >= kStats) return;
+// The blocks' sums, block k adding sum k in block order (at most kMaxBatch
+// blocks): one thread per SM, a chain of dependent FP64 additions.
+__global__ void __launch_bounds__(256) k_stats_final(const double *part, int nblk, double *out) {
+  __shared__ double sh[kMaxBatch];
+  const int k = blockIdx.x;
+  for (int b = threadIdx.x; b < nblk; b += blockDim.x) sh[b] = part[(int64_t)b * kStats + k];
+  __syncthreads();
+  if (threadIdx.x) return;
   double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += part[(int64_t)b * kStats + k];
+#pragma unroll 8
+  for (int b = 0; b < nblk; ++b) s += sh[b];
   out[k] = s;
 }
 
@@ -1047,7 +1173,7 @@ pl_status fit_start(const float *rec, int64_t nrec, float *w, const pl_train_opt
                     const TrainWs &W, cudaStream_t s) {
   const int nblk = (int)std::min<int64_t>(kMaxBatch, std::max<int64_t>(1, (nrec + 255) / 256));
   k_rec_stats<<<nblk, 256, 0, s>>>(rec, nrec, W.spart);
-  k_stats_final<<<1, 64, 0, s>>>(W.spart, nblk, W.sout);
+  k_stats_final<<<kStats, 256, 0, s>>>(W.spart, nblk, W.sout);
   note_launch();
   note_launch();
   double S[kStats];
@@ -1127,16 +1253,19 @@ pl_status pl_learned_train(const float *rec, int64_t nrec, float *w, const pl_tr
   const int bt = (int)std::min<int64_t>(o->batch_tiles, nfull);
   const int64_t spe = nfull / bt;
   const int64_t total = (int64_t)o->epochs * spe;
-  std::vector<int32_t> order((size_t)nfull);
-  const int rgrid = (kPart - kTH + 127) / 128;
-  int64_t step = 0;
-  for (int ep = 0; ep < o->epochs; ++ep) {
+  std::vector<int32_t> orders[2] = {std::vector<int32_t>((size_t)nfull), std::vector<int32_t>((size_t)nfull)};
+  auto shuffle = [&](int ep) {
+    std::vector<int32_t> &order = orders[ep & 1];
     for (int64_t i = 0; i < nfull; ++i) order[(size_t)i] = (int32_t)i;
     for (int64_t i = nfull - 1; i > 0; --i) {
       const uint64_t j = splitmix(o->seed, ((uint64_t)ep << 40) + (uint64_t)i) % (uint64_t)(i + 1);
       std::swap(order[(size_t)i], order[(size_t)j]);
     }
-    TRY(cudaMemcpyAsync(W.tiles, order.data(), (size_t)nfull * 4, cudaMemcpyHostToDevice, s));
+  };
+  int64_t step = 0;
+  shuffle(0);
+  for (int ep = 0; ep < o->epochs; ++ep) {
+    TRY(cudaMemcpyAsync(W.tiles, orders[ep & 1].data(), (size_t)nfull * 4, cudaMemcpyHostToDevice, s));
     TRY(cudaMemsetAsync(W.loss, 0, 8, s));
     for (int64_t k = 0; k < spe; ++k, ++step) {
       const double lr = o->lr_min + 0.5 * (o->lr - o->lr_min) *
@@ -1144,16 +1273,16 @@ pl_status pl_learned_train(const float *rec, int64_t nrec, float *w, const pl_tr
       const double t = (double)(step + 1);
       k_train_tile<<<bt, kTile, kSmemTrain, s>>>(rec, nrec, W.tiles + k * bt, 0,
                                                 1.f / (float)(bt * kTile), w, W.part, status);
-      k_reduce_parts<<<rgrid, 128, 0, s>>>(W.part, bt, W.acc, 1);
-      k_adam<<<rgrid, 128, 0, s>>>(W.acc, w, W.m, W.v, (float)lr, (float)o->beta1,
-                                   (float)o->beta2, (float)o->eps,
-                                   (float)(1.0 - std::pow(o->beta1, t)),
-                                   (float)(1.0 - std::pow(o->beta2, t)), W.loss);
-      note_launch();
+      k_adam<<<kPartGrid, 32 * kSegs, 0, s>>>(W.part, bt, w, W.m, W.v, (float)lr, (float)o->beta1,
+                                              (float)o->beta2, (float)o->eps,
+                                              (float)(1.0 - std::pow(o->beta1, t)),
+                                              (float)(1.0 - std::pow(o->beta2, t)), W.loss);
       note_launch();
       note_launch();
     }
     TRY(cudaGetLastError());
+    // the next epoch's order, in the other buffer, while this epoch runs
+    if (ep + 1 < o->epochs) shuffle(ep + 1);
     double l = 0.0;
     int sw = 0;
     TRY(cudaMemcpyAsync(&l, W.loss, 8, cudaMemcpyDeviceToHost, s));
@@ -1177,12 +1306,11 @@ pl_status pl_learned_loss(const float *rec, int64_t nrec, const float *w, void *
   int *status = reinterpret_cast<int *>(W.spart);
   TRY(cudaMemsetAsync(status, 0, 4, s));
   const int64_t ntiles = (nrec + kTile - 1) / kTile;
-  const int rgrid = (kPart - kTH + 127) / 128;
   for (int64_t t0 = 0; t0 < ntiles; t0 += kMaxBatch) {
     const int nb = (int)std::min<int64_t>(kMaxBatch, ntiles - t0);
     k_train_tile<<<nb, kTile, kSmemTrain, s>>>(rec, nrec, nullptr, t0, (float)(1.0 / (double)nrec), w,
                                                W.part, status);
-    k_reduce_parts<<<rgrid, 128, 0, s>>>(W.part, nb, W.acc, t0 == 0);
+    k_reduce_parts<<<kPartGrid, 32 * kSegs, 0, s>>>(W.part, nb, W.acc, t0 == 0);
     note_launch();
     note_launch();
   }
