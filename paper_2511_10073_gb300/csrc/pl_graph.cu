@@ -827,6 +827,12 @@ pl_status build_static(pl_graph *g, const pl_netlist *nl, const pl_params *p, cu
   g->nbx = p->nbx;
   g->nby = p->nby;
   g->NB = p->nbx * p->nby;
+  int nx = (int)floor(p->det_ratio * (double)g->nbx), ny = (int)floor(p->det_ratio * (double)g->nby);
+  if (nx < 1) nx = 1;
+  if (ny < 1) ny = 1;
+  g->hx = (nx - 1) / 2;
+  g->hy = (ny - 1) / 2;
+  g->W = (2 * g->hx + 1) * (2 * g->hy + 1);
   g->have_hints = false;
   g->stream = s;
 
@@ -1006,10 +1012,8 @@ pl_status build_static(pl_graph *g, const pl_netlist *nl, const pl_params *p, cu
   }
   TRY((segmented_sort<uint32_t, MODE_MERGE>(keys, row_off, Nst, npre, cnt, mcol, mval,
                                             g->tmp[3].p, s, maxrow)));
-  TRY(ensure(g->srp, (size_t)(Nst + 1) * 8));
-  TRY((exclusive_scan<int32_t, int64_t>(cnt, P<int64_t>(g->srp), Nst, stmp, s)));
   {
-    pl_status ls = prepare_static_layout(g, s);
+    pl_status ls = prepare_static_layout(g, cnt, s);
     if (ls != PL_OK) return ls;
   }
   TRY(ensure(g->base_w, (size_t)C * 8 + 16));
@@ -1067,11 +1071,6 @@ pl_status build_static(pl_graph *g, const pl_netlist *nl, const pl_params *p, cu
   g->wb = (g->xh - g->xl) / (double)g->nbx;
   g->hb = (g->yh - g->yl) / (double)g->nby;
   g->abin = g->wb * g->hb;
-  int nx = (int)floor(p->det_ratio * (double)g->nbx), ny = (int)floor(p->det_ratio * (double)g->nby);
-  if (nx < 1) nx = 1;
-  if (ny < 1) ny = 1;
-  g->hx = (nx - 1) / 2;
-  g->hy = (ny - 1) / 2;
   TRY(ensure(g->nkind, (size_t)N + 16));
   TRY(ensure(g->fixedp, (size_t)N * 8 + 16));
   TRY(ensure(g->bounds, (size_t)N * 16 + 16));
@@ -1168,11 +1167,8 @@ pl_status build_static(pl_graph *g, const pl_netlist *nl, const pl_params *p, cu
   TRY(cudaEventRecord(g->ev_join, s2));
   TRY(cudaStreamWaitEvent(s, g->ev_join, 0));
   TRY(cudaGetLastError());
-  {
-    int64_t nnz;  // read with the build's final synchronisation
-    TRY(d2h(&nnz, P<int64_t>(g->srp) + Nst, 1, s));
-    g->nnz_static = (uint64_t)nnz;
-  }
+  TRY(cudaStreamSynchronize(s));
+  g->nnz_static = g->st.nnz_s + g->st.nnz_l;
   (void)kMaxNetPins;
   {
     pl_status fs = take_filter_buffers(g);

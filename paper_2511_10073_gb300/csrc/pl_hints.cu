@@ -518,88 +518,315 @@ __global__ void k_dens_final(HintGeo G, int nlev, const int64_t *boff, const uin
   }
 }
 
-// ------------------------------------------------------- H6: row lengths
 __device__ __forceinline__ int win_count(int bx, int by, const HintGeo &G) {
   int nx = min(G.nbx - 1, bx + G.hx) - max(0, bx - G.hx) + 1;
   int ny = min(G.nby - 1, by + G.hy) - max(0, by - G.hy) + 1;
   return nx * ny;
 }
 
-// Per-row lengths of a split matrix.  Static mode: the st rows (hub when
-// longer than kLong).  Hint mode: the stored hm part of each row (a hint
-// cell's macro entries, a macro row's cells; bin rows store nothing, their
-// sums come from the window blocks); a row is a hub row when it is a virtual
-// node or its static entries, macro entries and window slots exceed kLong.
-// clen is the stored length the hub chunks cover (st part + hm part).
-__global__ void k_row_len(HintGeo G, int with_hints, const int64_t *srp, const uint8_t *hflag,
-                          const int32_t *cell_bin, const int32_t *n_ovl, const int64_t *moff,
-                          uint32_t *slen, uint64_t *llen, uint8_t *lflag, uint64_t *clen) {
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < G.N;
-       v += (long long)gridDim.x * blockDim.x) {
-    const long long sl = v < G.Nst ? srp[v + 1] - srp[v] : 0;
-    if (!with_hints) {
-      const bool hub = sl > kLong;
-      slen[v] = hub ? 0u : (uint32_t)sl;
-      llen[v] = hub ? (uint64_t)sl : 0ull;
-      lflag[v] = hub ? 1 : 0;
-      clen[v] = hub ? (uint64_t)sl : 0ull;
-      continue;
+// ------------------------------------------------- H6-H7: split layout
+// The layout of a split matrix in three launches: every row's place follows
+// from prefix sums over the rows of (short entries, hub entries, hub rows, hub
+// chunks), formed together.  k_lay_sum adds them per block of kLayRows rows,
+// k_lay_scan turns the block sums into offsets and totals (one block), and
+// k_lay_apply recomputes its rows' lengths and writes everything that depends
+// on them.  (As separate length, scan, pack and descriptor kernels this took
+// 14 launches and two reads of sizes by the host.)
+struct RowLen {
+  uint32_t s;      // short-region length (0 for hub rows)
+  uint64_t l, cl;  // hub-region length, chunked length of a hub row (st part + this matrix's part)
+  bool hub;
+};
+struct LayIn {
+  HintGeo G;
+  const int32_t *cnt;  // static matrix: row lengths; nullptr: hint matrix
+  const int64_t *srp;  // hint matrix: static row pointers
+  const uint8_t *hflag;
+  const int32_t *cell_bin, *n_ovl;
+  const int64_t *moff;
+  int may;  // static matrix: rows longer than this may become hub rows of the hint matrix
+};
+// Totals of a layout (device and host); may_*: static rows beyond LayIn::may
+// that are no hub rows, and their entries.
+struct LayTotals {
+  unsigned long long s, l, may_entries;
+  uint32_t f, c, may_rows, pad;
+};
+
+// Lengths of row v of a split matrix.  Static matrix: hub when longer than
+// kLong.  Hint matrix: the stored hm part of each row (a hint cell's macro
+// entries, a macro row's cells; bin rows store nothing, their sums come from
+// the window blocks); a row is a hub row when it is a virtual node or its static
+// entries, macro entries and window slots exceed kLong.
+template <bool HINT>
+__device__ __forceinline__ RowLen row_len(const LayIn &A, long long v) {
+  const HintGeo &G = A.G;
+  RowLen r{0u, 0ull, 0ull, false};
+  if (v >= G.N) return r;
+  if (!HINT) {
+    const uint32_t sl = v < G.Nst ? (uint32_t)A.cnt[v] : 0u;
+    r.hub = sl > (uint32_t)kLong;
+    if (r.hub) r.l = r.cl = sl;
+    else r.s = sl;
+    return r;
+  }
+  const long long sl = v < G.Nst ? A.srp[v + 1] - A.srp[v] : 0;
+  long long hl = 0, ws = 0;
+  bool virt = false;
+  if (v < G.C && A.hflag[v]) {
+    const int b = A.cell_bin[v];
+    hl = A.n_ovl[v];
+    ws = win_count(b % G.nbx, b / G.nbx, G);
+  } else if (v >= G.mv0 && v < G.bn0) {
+    hl = A.moff[v - G.mv0 + 1] - A.moff[v - G.mv0];
+    virt = true;
+  } else if (v >= G.bn0) {
+    virt = true;
+  }
+  r.hub = virt || sl + hl + ws > kLong;
+  if (r.hub) {
+    r.l = (uint64_t)hl;
+    r.cl = (uint64_t)(sl + hl);
+  } else {
+    r.s = (uint32_t)hl;
+  }
+  return r;
+}
+__device__ __forceinline__ uint32_t row_chunks(uint64_t cl) {
+  return cl == 0 ? 1u : (uint32_t)((cl + kChunk - 1) / kChunk);
+}
+
+constexpr int kLayPer = 8;                 // rows per lane (a warp: 256 consecutive rows)
+constexpr int kLayRows = 256 * kLayPer;    // rows per block of 256 threads
+struct LaySum {
+  unsigned long long s, l;
+  uint32_t f, c;
+};
+
+// This warp's sums over its rows (every lane gets them); sv, hubs: the lane's
+// short lengths and hub bits.
+template <bool HINT>
+__device__ __forceinline__ LaySum warp_rows(const LayIn &A, long long v0, uint32_t *sv,
+                                            uint32_t *hubs, unsigned long long *may_rows,
+                                            unsigned long long *may_entries) {
+  const int lane = threadIdx.x & 31;
+  LaySum t{0ull, 0ull, 0u, 0u};
+  *hubs = 0u;
+#pragma unroll
+  for (int k = 0; k < kLayPer; ++k) {
+    const RowLen r = row_len<HINT>(A, v0 + 32 * k + lane);
+    sv[k] = r.s;
+    t.s += r.s;
+    if (!HINT && v0 + 32 * k + lane < A.G.Nst && !r.hub && (int)r.s > A.may) {
+      ++*may_rows;
+      *may_entries += r.s;
     }
-    long long hl = 0, ws = 0;
-    bool virt = false;
-    if (v < G.C && hflag[v]) {
-      int b = cell_bin[v];
-      hl = n_ovl[v];
-      ws = win_count(b % G.nbx, b / G.nbx, G);
-    } else if (v >= G.mv0 && v < G.bn0) {
-      hl = moff[v - G.mv0 + 1] - moff[v - G.mv0];
-      virt = true;
-    } else if (v >= G.bn0) {
-      virt = true;
+    if (r.hub) {
+      *hubs |= 1u << k;
+      t.l += r.l;
+      t.f += 1u;
+      t.c += row_chunks(r.cl);
     }
-    const bool hub = virt || sl + hl + ws > kLong;
-    slen[v] = hub ? 0u : (uint32_t)hl;
-    llen[v] = hub ? (uint64_t)hl : 0ull;
-    lflag[v] = hub ? 1 : 0;
-    clen[v] = hub ? (uint64_t)(sl + hl) : 0ull;
+  }
+  t.s = warp_sum(t.s);
+  if (__any_sync(0xffffffffu, *hubs != 0u)) {
+    t.l = warp_sum(t.l);
+    t.f = warp_sum(t.f);
+    t.c = warp_sum(t.c);
+  }
+  return t;
+}
+
+template <bool HINT>
+__global__ void __launch_bounds__(256) k_lay_sum(LayIn A, LaySum *bsum, LayTotals *tot) {
+  __shared__ LaySum w[8];
+  uint32_t sv[kLayPer], hubs;
+  unsigned long long mr = 0, me = 0;
+  const int wid = threadIdx.x >> 5;
+  const LaySum t = warp_rows<HINT>(A, (long long)blockIdx.x * kLayRows + wid * 32 * kLayPer, sv, &hubs, &mr, &me);
+  if ((threadIdx.x & 31) == 0) w[wid] = t;
+  if (!HINT) {
+    mr = warp_sum(mr);
+    if (mr) {  // the same in every lane
+      me = warp_sum(me);
+      if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&tot->may_rows, (uint32_t)mr);
+        atomicAdd(&tot->may_entries, me);
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x) return;
+  LaySum a = w[0];
+  for (int k = 1; k < 8; ++k) {
+    a.s += w[k].s;
+    a.l += w[k].l;
+    a.f += w[k].f;
+    a.c += w[k].c;
+  }
+  bsum[blockIdx.x] = a;
+}
+
+// Exclusive scan of the block sums in place, totals to tot (one block).
+__global__ void __launch_bounds__(1024) k_lay_scan(int nblk, LaySum *bsum, LayTotals *tot) {
+  __shared__ LaySum w[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  auto add = [](LaySum &x, const LaySum &y) {
+    x.s += y.s;
+    x.l += y.l;
+    x.f += y.f;
+    x.c += y.c;
+  };
+  auto up = [&](LaySum x) {  // inclusive scan over the warp
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      LaySum y;
+      y.s = __shfl_up_sync(0xffffffffu, x.s, d);
+      y.l = __shfl_up_sync(0xffffffffu, x.l, d);
+      y.f = __shfl_up_sync(0xffffffffu, x.f, d);
+      y.c = __shfl_up_sync(0xffffffffu, x.c, d);
+      if (lane >= d) add(x, y);
+    }
+    return x;
+  };
+  LaySum carry{0ull, 0ull, 0u, 0u};
+  for (int b0 = 0; b0 < nblk; b0 += 1024) {
+    const int b = b0 + (int)threadIdx.x;
+    LaySum v{0ull, 0ull, 0u, 0u};
+    if (b < nblk) v = bsum[b];
+    const LaySum x = up(v);
+    if (lane == 31) w[wid] = x;
+    __syncthreads();
+    if (wid == 0) w[lane] = up(w[lane]);
+    __syncthreads();
+    LaySum off = carry;
+    if (wid) add(off, w[wid - 1]);
+    if (b < nblk) {
+      LaySum o = off;
+      o.s += x.s - v.s;
+      o.l += x.l - v.l;
+      o.f += x.f - v.f;
+      o.c += x.c - v.c;
+      bsum[b] = o;
+    }
+    add(carry, w[31]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    tot->s = carry.s;
+    tot->l = carry.l;
+    tot->f = carry.f;
+    tot->c = carry.c;
   }
 }
 
-__global__ void k_layout_long(int64_t N, const uint8_t *lflag, const int32_t *lscan,
-                              const uint64_t *lpos, const uint64_t *clen, uint64_t nnz_s,
-                              int32_t *lrow, uint64_t *lptr, int32_t *longidx,
-                              int32_t *nchunk_of) {
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N;
-       v += (long long)gridDim.x * blockDim.x) {
-    if (lflag[v]) {
-      int li = lscan[v];
-      lrow[li] = (int32_t)v;
-      lptr[li] = nnz_s + lpos[v];
-      longidx[v] = li;
-      const uint64_t len = clen[v];
-      nchunk_of[li] = len == 0 ? 1 : (int32_t)((len + kChunk - 1) / kChunk);
-    } else {
-      longidx[v] = -1;
-    }
-    if (v == N - 1) {
-      int nl = lscan[N];
-      lptr[nl] = nnz_s + lpos[N];
-    }
+// What the layout writes.  Short-row pointers carry the hub flag of each row in
+// bit 31 and are padded with the end offset, so that aligned reads may go a few
+// rows past N.  Hub rows get their node, their entries' place, their chunks and
+// the places of their st and hm pieces (see SpMat): the static matrix's own hub
+// region, or for the hint matrix the row's st part (short or hub region of st)
+// and its hm hub part.
+struct LayOut {
+  uint32_t *rp;
+  int64_t *srp;  // static matrix: the row pointers of all static rows
+  int32_t *longidx, *lrow, *lchunk, *chunk_lr;
+  uint64_t *lptr, *lsb, *lhb;
+  uint32_t *lsl, *lhl;
+  const uint32_t *st_rp;
+  const int32_t *st_longidx;
+  const uint64_t *st_lptr;
+};
+// Rows alone (rp, srp, longidx): what is needed before the hub arrays' sizes
+// are known.  HUBS: the hub arrays too.
+template <bool HINT, bool ROWS, bool HUBS>
+__global__ void __launch_bounds__(256) k_lay_apply(LayIn A, LayOut O, const LaySum *boff,
+                                                   const LayTotals *tot) {
+  __shared__ LaySum w[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const long long v0 = (long long)blockIdx.x * kLayRows + wid * 32 * kLayPer;
+  uint32_t sv[kLayPer], hubs;
+  unsigned long long mr = 0, me = 0;
+  const LaySum t = warp_rows<HINT>(A, v0, sv, &hubs, &mr, &me);
+  if (lane == 0) w[wid] = t;
+  __syncthreads();
+  LaySum o = boff[blockIdx.x];
+  for (int k = 0; k < wid; ++k) {
+    o.s += w[k].s;
+    o.l += w[k].l;
+    o.f += w[k].f;
+    o.c += w[k].c;
   }
-}
-
-__global__ void k_chunk_owner(int32_t nlong, const int32_t *lchunk, int32_t *chunk_lr) {
-  for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nlong; l += gridDim.x * blockDim.x)
-    for (int c = lchunk[l]; c < lchunk[l + 1]; ++c) chunk_lr[c] = l;
-}
-
-// Short-row pointers with the hub flag of each row in bit 31; padded with the
-// end offset so that aligned bulk copies may read a few entries past N.
-__global__ void k_rp_pack(const uint64_t *s64, const uint8_t *lflag, int64_t N, uint32_t *rp) {
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v <= N + kRpPad;
-       v += (long long)gridDim.x * blockDim.x) {
-    if (v < N) rp[v] = (uint32_t)s64[v] | (lflag[v] ? kHubFlag : 0u);
-    else rp[v] = (uint32_t)s64[N];
+  const long long N = A.G.N;
+  const unsigned long long ns = tot->s;
+#pragma unroll
+  for (int k = 0; k < kLayPer; ++k) {
+    const long long v = v0 + 32 * k + lane;
+    const bool hub = hubs >> k & 1u;
+    uint32_t x = sv[k];  // inclusive scan of the short lengths (at most 128 each)
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, d);
+      if (lane >= d) x += y;
+    }
+    const unsigned long long so = o.s + x - sv[k];
+    const unsigned hm = __ballot_sync(0xffffffffu, hub);
+    uint64_t lo = o.l;
+    uint32_t li = o.f, co = o.c;
+    if (hm) {  // warp-uniform
+      const RowLen r = hub ? row_len<HINT>(A, v) : RowLen{0u, 0ull, 0ull, false};
+      const uint32_t nc = hub ? row_chunks(r.cl) : 0u;
+      unsigned long long xl = r.l;
+      uint32_t xc = nc;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const unsigned long long yl = __shfl_up_sync(0xffffffffu, xl, d);
+        const uint32_t yc = __shfl_up_sync(0xffffffffu, xc, d);
+        if (lane >= d) {
+          xl += yl;
+          xc += yc;
+        }
+      }
+      lo += xl - r.l;
+      li += __popc(hm & lt);
+      co += xc - nc;
+      if (HUBS && hub) {
+        const uint64_t at = ns + lo;
+        O.lrow[li] = (int32_t)v;
+        O.lptr[li] = at;
+        O.lchunk[li] = (int32_t)co;
+        for (uint32_t c = 0; c < nc; ++c) O.chunk_lr[co + c] = (int32_t)li;
+        if (!HINT) {
+          O.lsb[li] = at;
+          O.lsl[li] = (uint32_t)r.l;
+          O.lhb[li] = 0;
+          O.lhl[li] = 0;
+        } else {
+          const int sli = v < A.G.Nst ? O.st_longidx[v] : -1;
+          O.lsb[li] = sli >= 0 ? O.st_lptr[sli] : (uint64_t)(O.st_rp[v] & kOffMask);
+          O.lsl[li] = (uint32_t)(r.cl - r.l);
+          O.lhb[li] = at;
+          O.lhl[li] = (uint32_t)r.l;
+        }
+      }
+      o.l += __shfl_sync(0xffffffffu, xl, 31);
+      o.f += __popc(hm);
+      o.c += __shfl_sync(0xffffffffu, xc, 31);
+    }
+    if (ROWS && v < N) {
+      O.rp[v] = (uint32_t)so | (hub ? kHubFlag : 0u);
+      O.longidx[v] = hub ? (int32_t)li : -1;
+    }
+    if (ROWS && !HINT && v <= A.G.Nst) O.srp[v] = (int64_t)(so + lo);
+    o.s += __shfl_sync(0xffffffffu, x, 31);
+  }
+  if (blockIdx.x != gridDim.x - 1 || threadIdx.x > kRpPad) return;
+  if (ROWS) {
+    O.rp[N + threadIdx.x] = (uint32_t)ns;
+  }
+  if (HUBS && threadIdx.x == 0) {
+    O.lptr[tot->f] = ns + tot->l;
+    O.lchunk[tot->f] = (int32_t)tot->c;
   }
 }
 
@@ -607,32 +834,6 @@ __global__ void k_u64_to_u32(const uint64_t *a, uint32_t *b, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     b[i] = (uint32_t)a[i];
-}
-
-// st and hm pieces of every hub row (see SpMat).  Static matrix: its own hub
-// region only.  Hint matrix: the row's st part (short or hub region of st) and
-// its hm hub part.
-__global__ void k_hub_desc(int32_t nlong, int with_hints, const int32_t *lrow,
-                           const uint64_t *lptr, const int64_t *srp, int64_t Nst,
-                           const uint32_t *st_rp, const int32_t *st_longidx,
-                           const uint64_t *st_lptr, uint64_t *lsb, uint32_t *lsl, uint64_t *lhb,
-                           uint32_t *lhl) {
-  for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nlong; l += gridDim.x * blockDim.x) {
-    if (!with_hints) {
-      lsb[l] = lptr[l];
-      lsl[l] = (uint32_t)(lptr[l + 1] - lptr[l]);
-      lhb[l] = 0;
-      lhl[l] = 0;
-      continue;
-    }
-    const int64_t v = lrow[l];
-    const long long sl = v < Nst ? srp[v + 1] - srp[v] : 0;
-    const int sli = v < Nst ? st_longidx[v] : -1;
-    lsb[l] = sli >= 0 ? st_lptr[sli] : (uint64_t)(st_rp[v] & kOffMask);
-    lsl[l] = (uint32_t)sl;
-    lhb[l] = lptr[l];
-    lhl[l] = (uint32_t)(lptr[l + 1] - lptr[l]);
-  }
 }
 
 // ------------------------------------------------------- H9: row assembly
@@ -1058,10 +1259,11 @@ __global__ void k_blocks_to_chunks(long long nthreads, int W, const int32_t *bch
 // (sorted by id), with the weights copied from the cells' own entries, so the
 // matrix is exactly symmetric.  Degree partials per chunk.
 __global__ void __launch_bounds__(256) k_hub_chunks(
-    HintGeo G, int wdtype, int32_t nchunks, const int32_t *chunk_lr, const int32_t *lrow,
+    HintGeo G, int wdtype, const uint32_t *pnchunks, const int32_t *chunk_lr, const int32_t *lrow,
     const uint64_t *lptr, const int32_t *lchunk, const int64_t *moff, const uint32_t *mlist,
     const int32_t *n_ovl, const uint64_t *mac_base, int32_t *col, void *w, dfl *cpart) {
   __shared__ dfl red[2][8];
+  const int nchunks = (int)*pnchunks;
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const int l = chunk_lr[c];
     const int64_t v = lrow[l];
@@ -1106,11 +1308,12 @@ __global__ void __launch_bounds__(256) k_hub_chunks(
 
 // Degrees of virtual rows (warp per row): a macro row from its chunk
 // partials, a bin row from the window blocks' degree partials per chunk.
-__global__ void k_hub_finalize(HintGeo G, BinGeo B, int32_t nlong, const int32_t *lrow,
+__global__ void k_hub_finalize(HintGeo G, BinGeo B, const uint32_t *pnlong, const int32_t *lrow,
                                const int32_t *lchunk, const dfl *cpart, const int32_t *bchunk,
                                const float4 *bdeg,
                                dfl *dsum, dfl *psum) {
   const int lane = threadIdx.x & 31;
+  const long long nlong = *pnlong;
   for (long long l = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; l < nlong;
        l += ((long long)gridDim.x * blockDim.x) >> 5) {
     const int64_t v = lrow[l];
@@ -1176,8 +1379,9 @@ __global__ void k_coef(int64_t N, const dfl *dsum, const double *lam, float *c32
   }
 }
 
-__global__ void k_coef_long(int32_t nlong, const int32_t *lrow, const dfl *dsum,
+__global__ void k_coef_long(const uint32_t *pnlong, const int32_t *lrow, const dfl *dsum,
                             const double *lam, double *c64) {
+  const int nlong = (int)*pnlong;
   for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nlong; l += gridDim.x * blockDim.x) {
     double d = df_to_d(dsum[lrow[l]]);
     c64[l] = 1.0 - d * lam[1];
@@ -1264,116 +1468,172 @@ static BinGeo make_bingeo(const pl_graph *g) {
   return B;
 }
 
-// Layout of a split matrix from per-row lengths already in g->slen/llen/lflag.
-// Layout of a split matrix from per-row lengths in g->slen/llen/clen and
-// hub flags in g->hubf.
-static pl_status layout(pl_graph *g, SpMat &m, int with_hints, cudaStream_t s) {
-  const int64_t N = g->N;
-  m.N = N;
-  void *stmp;
-  TRY(ensure(g->tmp[7], scan_tmp_bytes(N + 1) + 4096));
-  stmp = g->tmp[7].p;
-  TRY(ensure(g->lay[0], (size_t)(N + 1) * 8 + 256));
-  uint64_t *s64 = P<uint64_t>(g->lay[0]);
-  TRY((exclusive_scan<uint32_t, uint64_t>(P<uint32_t>(g->slen), s64, N, stmp, s)));
-  TRY(ensure(g->lay[1], (size_t)(N + 1) * 8 + 256));
-  uint64_t *lpos = P<uint64_t>(g->lay[1]);
-  TRY((exclusive_scan<uint64_t, uint64_t>(P<uint64_t>(g->llen), lpos, N, stmp, s)));
-  TRY(ensure(g->lflag, (size_t)(N + 1) * 4 + 256));
-  int32_t *lscan = P<int32_t>(g->lflag);
-  TRY((exclusive_scan<uint8_t, int32_t>(P<uint8_t>(g->hubf), lscan, N, stmp, s)));
-  uint64_t tot[2];
-  int32_t nl;
-  {
-    const D2H it[3] = {{&tot[0], s64 + N, 8}, {&tot[1], lpos + N, 8}, {&nl, lscan + N, 4}};
-    TRY(d2h_many(g->stage, it, 3, s));
+// First part of a layout: the block sums, offsets and totals (device), in
+// g->lay[0] and g->lay[1].
+static pl_status lay_sums(pl_graph *g, const LayIn &A, cudaStream_t s, LaySum **bsum,
+                          LayTotals **tot, int *nblk) {
+  *nblk = (int)((g->N + kLayRows - 1) / kLayRows);
+  TRY(ensure(g->lay[0], (size_t)*nblk * sizeof(LaySum) + 256));
+  TRY(ensure(g->lay[1], sizeof(LayTotals) + 256));
+  *bsum = P<LaySum>(g->lay[0]);
+  *tot = P<LayTotals>(g->lay[1]);
+  if (A.cnt) {
+    TRY(cudaMemsetAsync(*tot, 0, sizeof(LayTotals), s));
+    k_lay_sum<false><<<*nblk, 256, 0, s>>>(A, *bsum, *tot);
+  } else {
+    k_lay_sum<true><<<*nblk, 256, 0, s>>>(A, *bsum, *tot);
   }
-  if (tot[0] + kPad >= (uint64_t)kOffMask || tot[0] + tot[1] >= (1ull << 40)) {
-    set_error("graph too large for the 31-bit short-row layout (%llu entries)",
-              (unsigned long long)tot[0]);
-    return PL_ERR_UNSUPPORTED;
-  }
-  m.nnz_s = tot[0];
-  m.nnz_l = tot[1];
-  m.nlong = nl;
-  m.wbytes = g->wdtype == PL_W_BF16 ? 2 : 4;
-  TRY(ensure(m.rp_s, (size_t)(N + 1 + kRpPad) * 4));
-  k_rp_pack<<<grid_for(N + 1 + kRpPad, 256), 256, 0, s>>>(s64, P<uint8_t>(g->hubf), N,
-                                                         P<uint32_t>(m.rp_s));
   note_launch();
-  const uint64_t cap = m.nnz_s + m.nnz_l + kPad;
+  k_lay_scan<<<1, 1024, 0, s>>>(*nblk, *bsum, *tot);
+  note_launch();
+  return PL_OK;
+}
+
+static bool lay_too_large(uint64_t ns, uint64_t nl) {
+  if (ns + kPad < (uint64_t)kOffMask && ns + nl < (1ull << 40)) return false;
+  set_error("graph too large for the 31-bit short-row layout (%llu entries)",
+            (unsigned long long)ns);
+  return true;
+}
+
+// The hub arrays for nl hub rows and nc chunks.
+static cudaError_t lay_hub_arrays(SpMat &m, size_t nl, size_t nc) {
+  cudaError_t e = ensure(m.lrow, nl * 4 + 16);
+  if (e == cudaSuccess) e = ensure(m.lptr, (nl + 1) * 8);
+  if (e == cudaSuccess) e = ensure(m.lsb, nl * 8 + 16);
+  if (e == cudaSuccess) e = ensure(m.lhb, nl * 8 + 16);
+  if (e == cudaSuccess) e = ensure(m.lsl, nl * 4 + 16);
+  if (e == cudaSuccess) e = ensure(m.lhl, nl * 4 + 16);
+  if (e == cudaSuccess) e = ensure(m.lchunk, (nl + 1) * 4);
+  if (e == cudaSuccess) e = ensure(m.chunk_lr, nc * 4 + 16);
+  if (e == cudaSuccess) e = ensure(m.c64l, nl * 8 + 16);
+  return e;
+}
+static size_t lay_hub_bytes(size_t nl, size_t nc) {
+  return nl * 48 + nc * 4 + 9 * 256 + 256;
+}
+
+static LayOut lay_out(pl_graph *g, SpMat &m) {
+  LayOut O;
+  O.rp = P<uint32_t>(m.rp_s);
+  O.srp = P<int64_t>(g->srp);
+  O.longidx = P<int32_t>(m.longidx);
+  O.lrow = P<int32_t>(m.lrow);
+  O.lchunk = P<int32_t>(m.lchunk);
+  O.chunk_lr = P<int32_t>(m.chunk_lr);
+  O.lptr = P<uint64_t>(m.lptr);
+  O.lsb = P<uint64_t>(m.lsb);
+  O.lhb = P<uint64_t>(m.lhb);
+  O.lsl = P<uint32_t>(m.lsl);
+  O.lhl = P<uint32_t>(m.lhl);
+  O.st_rp = P<uint32_t>(g->st.rp_s);
+  O.st_longidx = P<int32_t>(g->st.longidx);
+  O.st_lptr = P<uint64_t>(g->st.lptr);
+  return O;
+}
+
+// The entries' arrays (nnz of them and the spare ones, zeroed) and the arrays
+// over all rows.
+static pl_status lay_entries(pl_graph *g, SpMat &m, uint64_t nnz, cudaStream_t s) {
+  const int64_t N = g->N;
+  const uint64_t cap = nnz + kPad;
+  m.N = N;
+  m.wbytes = g->wdtype == PL_W_BF16 ? 2 : 4;
   TRY(ensure(m.col, cap * 4));
   TRY(ensure(m.w, cap * m.wbytes));
-  TRY(ensure(m.lrow, (size_t)nl * 4 + 16));
-  TRY(ensure(m.lptr, (size_t)(nl + 1) * 8));
-  TRY(ensure(m.lsb, (size_t)nl * 8 + 16));
-  TRY(ensure(m.lhb, (size_t)nl * 8 + 16));
-  TRY(ensure(m.lsl, (size_t)nl * 4 + 16));
-  TRY(ensure(m.lhl, (size_t)nl * 4 + 16));
-  TRY(ensure(m.longidx, (size_t)N * 4 + 16));
-  TRY(ensure(m.lchunk, (size_t)(nl + 1) * 4));
-  TRY(ensure(g->lay[3], (size_t)(nl + 1) * 4 + 256));
-  int32_t *nch = P<int32_t>(g->lay[3]);
-  k_layout_long<<<grid_for(N, 256), 256, 0, s>>>(N, P<uint8_t>(g->hubf), lscan, lpos,
-                                                 P<uint64_t>(g->clen), m.nnz_s,
-                                                 P<int32_t>(m.lrow), P<uint64_t>(m.lptr),
-                                                 P<int32_t>(m.longidx), nch);
-  note_launch();
-  if (nl == 0) {
-    TRY(cudaMemsetAsync(m.lchunk.p, 0, 4, s));
-    m.nchunks = 0;
-  } else {
-    TRY((exclusive_scan<int32_t, int32_t>(nch, P<int32_t>(m.lchunk), nl, stmp, s)));
-    int32_t nc;
-    TRY(d2h(&nc, P<int32_t>(m.lchunk) + nl, 1, s));
-    m.nchunks = nc;
-    k_hub_desc<<<grid_for(nl, 256), 256, 0, s>>>(
-        nl, with_hints, P<int32_t>(m.lrow), P<uint64_t>(m.lptr), P<int64_t>(g->srp), g->Nst,
-        P<uint32_t>(g->st.rp_s), P<int32_t>(g->st.longidx), P<uint64_t>(g->st.lptr),
-        P<uint64_t>(m.lsb), P<uint32_t>(m.lsl), P<uint64_t>(m.lhb), P<uint32_t>(m.lhl));
-    note_launch();
-  }
-  TRY(ensure(m.chunk_lr, (size_t)m.nchunks * 4 + 16));
-  if (nl) {
-    k_chunk_owner<<<grid_for(nl, 256), 256, 0, s>>>(nl, P<int32_t>(m.lchunk), P<int32_t>(m.chunk_lr));
-    note_launch();
-  }
   TRY(ensure(m.dsum, (size_t)N * 8 + 16));
   TRY(ensure(m.psum, (size_t)N * 8 + 16));
   TRY(ensure(m.c32, (size_t)N * 4 + 16));
-  TRY(ensure(m.c64l, (size_t)nl * 8 + 16));
   TRY(ensure(m.lam, 64));
-  size_t pbytes = (size_t)(m.nchunks + 1) * 6 * 8;
-  TRY(ensure(m.part, pbytes));
-  TRY(cudaMemsetAsync(P<char>(m.col) + (m.nnz_s + m.nnz_l) * 4, 0, kPad * 4, s));
-  TRY(cudaMemsetAsync(P<char>(m.w) + (m.nnz_s + m.nnz_l) * m.wbytes, 0, kPad * m.wbytes, s));
+  TRY(cudaMemsetAsync(P<char>(m.col) + nnz * 4, 0, kPad * 4, s));
+  TRY(cudaMemsetAsync(P<char>(m.w) + nnz * m.wbytes, 0, kPad * m.wbytes, s));
   return PL_OK;
 }
 
-static pl_status ensure_row_arrays(pl_graph *g) {
-  const int64_t N = g->N;
-  TRY(ensure(g->slen, (size_t)N * 4 + 16));
-  TRY(ensure(g->llen, (size_t)N * 8 + 16));
-  TRY(ensure(g->clen, (size_t)N * 8 + 16));
-  TRY(ensure(g->hubf, (size_t)N + 256));
-  return PL_OK;
+static void lay_totals(SpMat &m, const LayTotals &t) {
+  m.nnz_s = t.s;
+  m.nnz_l = t.l;
+  m.nlong = (int32_t)t.f;
+  m.nchunks = (int32_t)t.c;
 }
 
-// Layout of the static split matrix from the static row pointers; the
-// entries and degree sums are written by the static compaction.
-pl_status prepare_static_layout(pl_graph *g, cudaStream_t s) {
+// Layout of the static split matrix and the static row pointers from the row
+// lengths cnt; the entries and degree sums are written by the static
+// compaction.  Its totals are read with one synchronisation, after the row
+// pointers were launched.
+pl_status prepare_static_layout(pl_graph *g, const int32_t *cnt, cudaStream_t s) {
   const int64_t N = g->N;
-  HintGeo G{};
-  G.N = N;
-  G.Nst = g->Nst;
-  pl_status st = ensure_row_arrays(g);
+  LayIn A{};
+  A.G.N = N;
+  A.G.Nst = g->Nst;
+  A.cnt = cnt;
+  A.may = kLong - g->W - kMacroSlots;
+  LaySum *bsum;
+  LayTotals *tot, t;
+  int nblk;
+  pl_status st = lay_sums(g, A, s, &bsum, &tot, &nblk);
   if (st != PL_OK) return st;
-  k_row_len<<<grid_for(N, 256), 256, 0, s>>>(G, 0, P<int64_t>(g->srp), nullptr, nullptr, nullptr,
-                                             nullptr, P<uint32_t>(g->slen),
-                                             P<uint64_t>(g->llen), P<uint8_t>(g->hubf),
-                                             P<uint64_t>(g->clen));
+  SpMat &m = g->st;
+  TRY(ensure(m.rp_s, (size_t)(N + 1 + kRpPad) * 4));
+  TRY(ensure(m.longidx, (size_t)N * 4 + 16));
+  TRY(ensure(g->srp, (size_t)(g->Nst + 1) * 8));
+  k_lay_apply<false, true, false><<<nblk, 256, 0, s>>>(A, lay_out(g, m), bsum, tot);
   note_launch();
-  return layout(g, g->st, 0, s);
+  {
+    const D2H it[1] = {{&t, tot, sizeof(LayTotals)}};
+    TRY(d2h_many(g->stage, it, 1, s));
+  }
+  if (lay_too_large(t.s, t.l)) return PL_ERR_UNSUPPORTED;
+  lay_totals(m, t);
+  g->may_rows = t.may_rows;
+  g->may_entries = t.may_entries;
+  TRY(lay_hub_arrays(m, t.f, t.c));
+  if (t.f) {
+    k_lay_apply<false, false, true><<<nblk, 256, 0, s>>>(A, lay_out(g, m), bsum, tot);
+    note_launch();
+  } else {
+    TRY(cudaMemsetAsync(m.lchunk.p, 0, 4, s));
+  }
+  TRY(ensure(m.part, (size_t)(t.c + 1) * 16));
+  return lay_entries(g, m, t.s + t.l, s);
+}
+
+// Layout of the hint matrix for nml macro-cell overlaps, without a read by the
+// host where bounds on the hub rows and chunks fit the workspace: a short
+// static row can only become a hub row when it is longer than kLong less the
+// window slots and kMacroSlots macro entries (exact_ok: no cell has more), and
+// the static layout has counted those.  later: workspace bytes that the rest of
+// the build will ask for.  *nl_max, *nc_max: hub rows and chunks at most; the totals stay on the device (*tot) until the build's last read.
+static pl_status layout_hints(pl_graph *g, const LayIn &A, int64_t nml, bool exact_ok,
+                              size_t later, cudaStream_t s, LayTotals **tot, size_t *nl_max, size_t *nc_max) {
+  const int64_t N = g->N;
+  LaySum *bsum;
+  int nblk;
+  pl_status st = lay_sums(g, A, s, &bsum, tot, &nblk);
+  if (st != PL_OK) return st;
+  SpMat &m = g->hm;
+  TRY(ensure(m.rp_s, (size_t)(N + 1 + kRpPad) * 4));
+  TRY(ensure(m.longidx, (size_t)N * 4 + 16));
+  st = lay_entries(g, m, 2 * (uint64_t)nml, s);
+  if (st != PL_OK) return st;
+  size_t nl = (size_t)g->Mm + g->NB + g->st.nlong + g->may_rows;
+  size_t nc = nl + (size_t)((g->st.nnz_l + g->may_entries + 2 * (uint64_t)nml) / kChunk) + 1;
+  const Arena *ar = current_arena();
+  if (!exact_ok || (uint64_t)nml + kPad >= (uint64_t)kOffMask ||
+      lay_hub_bytes(nl, nc) + nc * 32 + later > ar->cap - ar->used) {
+    LayTotals t;
+    const D2H it[1] = {{&t, *tot, sizeof(LayTotals)}};
+    TRY(d2h_many(g->stage, it, 1, s));
+    if (lay_too_large(t.s, t.l)) return PL_ERR_UNSUPPORTED;
+    nl = t.f;
+    nc = t.c;
+  }
+  TRY(lay_hub_arrays(m, nl, nc));
+  k_lay_apply<true, true, true><<<nblk, 256, 0, s>>>(A, lay_out(g, m), bsum, *tot);
+  note_launch();
+  *nl_max = nl;
+  *nc_max = nc;
+  return PL_OK;
 }
 
 pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaStream_t s) {
@@ -1575,28 +1835,31 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   TRY(cudaEventRecord(g->ev_join, s2));
   TRY(cudaEventRecord(g->ev_join2, s3));
   // H6-H7: row lengths and layout
-  pl_status st = ensure_row_arrays(g);
-  if (st != PL_OK) return st;
-  k_row_len<<<grid_for(N, 256), 256, 0, s>>>(G, 1, P<int64_t>(g->srp), P<uint8_t>(g->hflag),
-                                             P<int32_t>(g->cell_bin), P<int32_t>(g->n_ovl),
-                                             P<int64_t>(g->moff), P<uint32_t>(g->slen),
-                                             P<uint64_t>(g->llen), P<uint8_t>(g->hubf),
-                                             P<uint64_t>(g->clen));
-  note_launch();
-  st = layout(g, g->hm, 1, s);
+  LayIn LA{};
+  LA.G = G;
+  LA.srp = P<int64_t>(g->srp);
+  LA.hflag = P<uint8_t>(g->hflag);
+  LA.cell_bin = P<int32_t>(g->cell_bin);
+  LA.n_ovl = P<int32_t>(g->n_ovl);
+  LA.moff = P<int64_t>(g->moff);
+  LayTotals *tot;
+  size_t nl_max, nc_max;
+  const int W = g->W;
+  const size_t wb = g->wdtype == PL_W_BF16 ? 2 : 4;
+  const long long nbc_max = nbl / kBinChunk + NB + 1;  // bin-row chunks at most (the grid size)
+  const size_t later = (size_t)C * (8 + W * wb + 4) + (size_t)(NB + 1) * 8 +
+                       (size_t)nbc_max * (4 + kBinChunk * W * wb + 32 * W) + 16 * 512;
+  pl_status st = layout_hints(g, LA, nml, cmem_ok || Mm == 0, later, s, &tot, &nl_max, &nc_max);
   if (st != PL_OK) return st;
   SpMat &m = g->hm;
   // H9: hint parts of cells (macro entries, window blocks) and degrees of
   // every real node
   TRY(ensure(g->mac_base, (size_t)C * 8 + 16));
-  const int W = (2 * g->hx + 1) * (2 * g->hy + 1);
-  g->W = W;
   TRY(ensure(g->hbw, (size_t)C * W * m.wbytes + 64));
   TRY(ensure(g->hbin, (size_t)C * 4 + 16));
   unsigned long long *counts = reinterpret_cast<unsigned long long *>(P<double>(m.lam) + 3);
   TRY(cudaMemsetAsync(counts, 0, 16, s));
-  TRY(cudaStreamWaitEvent(s, g->ev_join, 0));   // phi
-  TRY(cudaStreamWaitEvent(s, g->ev_join2, 0));  // the macro lists
+  TRY(cudaStreamWaitEvent(s, g->ev_join, 0));  // phi
   (g->wdtype == PL_W_BF16 ? k_assemble_hints<true> : k_assemble_hints<false>)
       <<<grid_for(g->Nst, 256), 256, 0, s>>>(
       G, exp_table(), P<uint32_t>(m.rp_s), P<int32_t>(m.longidx), P<uint64_t>(m.lptr),
@@ -1615,7 +1878,6 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   k_bin_chunk_count<<<grid_for(NB, 256), 256, 0, s>>>(NB, P<int64_t>(g->boff), P<int32_t>(g->tmp[6]));
   note_launch();
   TRY((exclusive_scan<int32_t, int32_t>(P<int32_t>(g->tmp[6]), P<int32_t>(g->bchunk), NB, stmp, s)));
-  const long long nbc_max = nbl / kBinChunk + NB + 1;  // chunks at most (the grid size)
   g->nbc_max = nbc_max;
   TRY(ensure(g->cown, (size_t)nbc_max * 4 + 256));
   k_chunk_bins<<<grid_for(nbc_max, 256), 256, 0, s>>>(NB, nbc_max, P<int32_t>(g->bchunk), P<int32_t>(g->cown));
@@ -1642,16 +1904,17 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
                                  P<int64_t>(g->boff), P<uint32_t>(g->blist), g->hbwq.p, nullptr,
                                  P<float4>(g->bdeg)));
   note_launch();
-  TRY(ensure(g->tmp[5], (size_t)(m.nchunks + 1) * 2 * sizeof(dfl) + 256));
+  TRY(ensure(g->tmp[5], (nc_max + 1) * 2 * sizeof(dfl) + 256));
   dfl *cpart = P<dfl>(g->tmp[5]);
-  if (m.nchunks) {
-    k_hub_chunks<<<m.nchunks < 152 * 32 ? m.nchunks : 152 * 32, 256, 0, s>>>(
-        G, g->wdtype, m.nchunks, P<int32_t>(m.chunk_lr), P<int32_t>(m.lrow), P<uint64_t>(m.lptr),
+  TRY(cudaStreamWaitEvent(s, g->ev_join2, 0));  // the macro lists
+  if (nc_max) {
+    k_hub_chunks<<<(int)(nc_max < 152 * 32 ? nc_max : 152 * 32), 256, 0, s>>>(
+        G, g->wdtype, &tot->c, P<int32_t>(m.chunk_lr), P<int32_t>(m.lrow), P<uint64_t>(m.lptr),
         P<int32_t>(m.lchunk), P<int64_t>(g->moff), P<uint32_t>(g->mlist), P<int32_t>(g->n_ovl),
         P<uint64_t>(g->mac_base), P<int32_t>(m.col), m.w.p, cpart);
     note_launch();
-    k_hub_finalize<<<grid_for((long long)m.nlong * 32, 256), 256, 0, s>>>(
-        G, B, m.nlong, P<int32_t>(m.lrow), P<int32_t>(m.lchunk), cpart, P<int32_t>(g->bchunk),
+    k_hub_finalize<<<grid_for((long long)nl_max * 32, 256), 256, 0, s>>>(
+        G, B, &tot->f, P<int32_t>(m.lrow), P<int32_t>(m.lchunk), cpart, P<int32_t>(g->bchunk),
         P<float4>(g->bdeg),
         P<dfl>(m.dsum), P<dfl>(m.psum));
     note_launch();
@@ -1665,16 +1928,19 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   note_launch();
   k_coef<<<grid_for(N, 256), 256, 0, s>>>(N, P<dfl>(m.dsum), P<double>(m.lam), P<float>(m.c32));
   note_launch();
-  if (m.nlong) {
-    k_coef_long<<<grid_for(m.nlong, 256), 256, 0, s>>>(m.nlong, P<int32_t>(m.lrow), P<dfl>(m.dsum),
+  if (nl_max) {
+    k_coef_long<<<grid_for((long long)nl_max, 256), 256, 0, s>>>(&tot->f, P<int32_t>(m.lrow), P<dfl>(m.dsum),
                                                         P<double>(m.lam), P<double>(m.c64l));
     note_launch();
   }
   TRY(cudaGetLastError());
   {
     unsigned long long ns[2] = {0, 0};
-    const D2H it[2] = {{hst, g->status.p, 32}, {ns, counts, 16}};
-    TRY(d2h_many(g->stage, it, 2, s));
+    LayTotals t;
+    const D2H it[3] = {{hst, g->status.p, 32}, {ns, counts, 16}, {&t, tot, sizeof(LayTotals)}};
+    TRY(d2h_many(g->stage, it, 3, s));
+    lay_totals(m, t);
+    TRY(ensure(m.part, (size_t)(t.c + 1) * 16));
     g->nslot = (int64_t)ns[0];
     g->nhint = (int64_t)ns[1];
   }

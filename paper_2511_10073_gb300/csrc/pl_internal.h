@@ -54,7 +54,7 @@ struct SpMat {
   Buf c64l;     // double [nlong] same, FP64, hub rows
   Buf lam;      // 8-byte words: lambda_up, 1/lambda_up (double), the raw max key, the
                 // count of window slots inside the grid and of hint cells (uint64)
-  Buf part;     // float4 [nchunks] hub partial sums (two double-floats)
+  Buf part;     // float4 [nchunks + 1] hub partial sums (two double-floats)
   int wbytes = 4;
 };
 
@@ -106,10 +106,8 @@ struct pl_graph {
   pl::Buf mtc, mtoff;  // per (macro, cell tile) counts and their scan (tiled macro lists)
   pl::Buf cmem;        // int32 [C * 8] each hint cell's macros (tiled macro lists)
   pl::Buf Db, phi;     // double [NB]
-  pl::Buf slen;        // uint32 [N] short-region length (0 for hub rows)
-  pl::Buf llen;        // uint64 [N] hub-region length (0 for short rows)
-  pl::Buf clen;        // uint64 [N] chunked length of hub rows
-  pl::Buf lflag;       // int32 [N+1] hub flag scan
+  // short static rows that may become hub rows of a hint matrix, and their entries
+  uint64_t may_rows = 0, may_entries = 0;
   pl::Buf mac_base;    // uint64 [C] entry offset of a cell's first macro entry
   // bin hints without stored columns: each hint cell's window block and the
   // bin rows as its transpose over the bucket lists
@@ -154,8 +152,7 @@ struct pl_graph {
   int occ_rows[2][2] = {{0, 0}, {0, 0}};
   int occ_rows4[2] = {0, 0};
   pl::Buf tmp[8];
-  pl::Buf lay[4];         // layout scratch (scans of row lengths, chunk counts)
-  pl::Buf hubf;           // uint8 [N] hub flags of a layout
+  pl::Buf lay[2];         // layout scratch (block sums, totals)
 };
 
 namespace pl {
@@ -167,8 +164,7 @@ __global__ void k_cell_area(int32_t C, const float *cw, const float *ch, double 
 template <typename F>
 void for_each_buf(pl_graph *g, int kind, F f) {
   Buf *hint[] = {&g->tmp[0], &g->tmp[1], &g->tmp[2], &g->tmp[3], &g->tmp[4], &g->tmp[5],
-                 &g->tmp[6], &g->tmp[7], &g->lay[0], &g->lay[1], &g->lay[2], &g->lay[3],
-                 &g->hubf, &g->slen, &g->llen, &g->clen, &g->lflag, &g->hubtmp, &g->cell_bin,
+                 &g->tmp[6], &g->tmp[7], &g->lay[0], &g->lay[1], &g->hubtmp, &g->cell_bin,
                  &g->n_ovl, &g->bcnt, &g->boff, &g->blist, &g->bcur, &g->mcnt, &g->moff,
                  &g->mlist, &g->mcur, &g->mtc, &g->mtoff, &g->cmem, &g->Db, &g->phi,
                  &g->mac_base, &g->hbw, &g->hbwq, &g->hbin, &g->bchunk, &g->cown, &g->bdeg,
@@ -200,7 +196,7 @@ pl_status build_static(pl_graph *g, const pl_netlist *nl, const pl_params *p, cu
 pl_status take_filter_buffers(pl_graph *g);
 double workspace_bound(const pl_netlist *nl, const pl_params *p);
 pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy, cudaStream_t s);
-pl_status prepare_static_layout(pl_graph *g, cudaStream_t s);
+pl_status prepare_static_layout(pl_graph *g, const int32_t *cnt, cudaStream_t s);
 pl_status run_init_signal(pl_graph *g, uint64_t seed, const float *xy0, float *xy, cudaStream_t s);
 pl_status run_gift(pl_graph *g, const pl_params *p, const float *in, float *out, cudaStream_t s);
 pl_status run_filter(pl_graph *g, const pl_params *p, const float *in, float *out, cudaStream_t s);

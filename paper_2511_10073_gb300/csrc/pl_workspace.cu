@@ -72,16 +72,11 @@ double workspace_bound(const pl_netlist *nl, const pl_params *p) {
   st.add(npre * 12 + 512);
   st.add(seg_b(Nst, npre));
   st.add((Nst + 1) * 8);
-  // static layout (row lengths, the split matrix)
+  // static layout (block sums and totals, the split matrix)
   const double nchunk_st = N + npre / kChunk + 1;
-  st.add(N * 4 + 16);
-  st.add(N * 8 + 16);
-  st.add(N * 8 + 16);
-  st.add(N + 256);
-  st.add(scan_b(N + 1));
-  st.add((N + 1) * 8 + 256);
-  st.add((N + 1) * 8 + 256);
-  st.add((N + 1) * 4 + 256);
+  const double lay_b = std::ceil(N / 2048.0) * 24 + 256;
+  st.add(lay_b);
+  st.add(512);
   st.add((N + 1 + kRpPad) * 4);
   st.add((npre + kPad) * 4);
   st.add((npre + kPad) * sw);
@@ -89,14 +84,13 @@ double workspace_bound(const pl_netlist *nl, const pl_params *p) {
   st.add((N + 1) * 8);                                            // lptr
   st.add(N * 4 + 16);                                             // longidx
   st.add((N + 1) * 4);                                            // lchunk
-  st.add((N + 1) * 4 + 256);                                      // chunk counts
   st.add(nchunk_st * 4 + 16);
   st.add(N * 8 + 16);
   st.add(N * 8 + 16);
   st.add(N * 4 + 16);
   st.add(N * 8 + 16);
   st.add(64);
-  st.add((nchunk_st + 1) * 48);
+  st.add((nchunk_st + 1) * 16);
   // baseWeight, hint flags, star weights, node tables, bins, macro geometry
   st.add(C * 8 + 16);
   st.add(C + 16);
@@ -162,13 +156,8 @@ double workspace_bound(const pl_netlist *nl, const pl_params *p) {
   }
   const double hm_cap = 2 * nml + kPad;
   const double nchunk_h = N + (npre + 2 * nml) / kChunk + 1;
-  h.add(N * 4 + 16);
-  h.add(N * 8 + 16);
-  h.add(N * 8 + 16);
-  h.add(N + 256);
-  h.add((N + 1) * 8 + 256);
-  h.add((N + 1) * 8 + 256);
-  h.add((N + 1) * 4 + 256);
+  h.add(lay_b);
+  h.add(512);
   h.add((N + 1 + kRpPad) * 4);
   h.add(hm_cap * 4);
   h.add(hm_cap * sw);
@@ -176,14 +165,13 @@ double workspace_bound(const pl_netlist *nl, const pl_params *p) {
   h.add((N + 1) * 8);
   h.add(N * 4 + 16);
   h.add((N + 1) * 4);
-  h.add((N + 1) * 4 + 256);
   h.add(nchunk_h * 4 + 16);
   h.add(N * 8 + 16);
   h.add(N * 8 + 16);
   h.add(N * 4 + 16);
   h.add(N * 8 + 16);
   h.add(64);
-  h.add((nchunk_h + 1) * 48);
+  h.add((nchunk_h + 1) * 16);
   h.add(C * 8 + 16);                 // macro entry offsets
   h.add(C * W * sw + 64);            // window blocks, cell order
   h.add((std::floor(nmov / kBinChunk) + NB + 1) * kBinChunk * W * sw + 64);  // chunks' window blocks
