@@ -1,15 +1,16 @@
 // A5: half-perimeter wirelength (the quality metric of Sec. VII-VIII):
 // sum over nets of (max - min) pin x + (max - min) pin y, pin = cell centre +
-// offset.  A thread takes a net of up to 32 pins (a warp stages the pins of 32
-// consecutive nets when they fit), a warp a net of up to 1024; each block then
-// spans the larger nets of its own range of nets, one at a time with all its
-// threads.  Pin positions and extrema are FP32 (min/max are exact); each net's
-// span is formed exactly and summed in double-float per thread, the threads'
-// sums in FP64.  Per-block sums go to the caller's workspace; the last block
-// to finish (ticket) adds them in a fixed order (strided over its threads,
-// then a fixed tree), so the result does not depend on scheduling.  A pin
-// whose cell index is out of range makes the result NaN (it is not
-// dereferenced).
+// offset.  A warp takes 32 consecutive nets at a time and brings their pins'
+// positions through shared memory in windows; a lane spans its own net there,
+// the warp together the part of a net of more than kHpwlLane pins; nets of more
+// than kHpwlWarpMax pins are left to the whole block.  Pin positions and
+// extrema are FP32 (min/max are exact); each net's span is formed exactly and
+// summed in double-float per thread, the threads' sums in FP64.  Per-block sums
+// go to the caller's workspace; the last block to finish (ticket) adds them in a
+// fixed order (strided over its threads, then a fixed tree), so the result does
+// not depend on scheduling.  A pin whose cell index is out of range makes the
+// result NaN (it is not dereferenced).
+#include <cmath>
 #include <mutex>
 
 #include "pl_internal.h"
@@ -18,23 +19,44 @@ namespace pl {
 
 constexpr int kHpwlThreads = 256;
 constexpr int kHpwlBlocks = 152 * 8;
-constexpr int kHpwlStage = 512;  // pins of one batch of 32 nets staged per warp
-constexpr int kHpwlWarpMax = 1024;  // longer nets are spanned by a whole block
+constexpr int kHpwlPerSm = 4;
+constexpr int kHpwlGrid = 152 * kHpwlPerSm;     // what is launched: one wave of resident blocks
+constexpr int kHpwlWin = 256;        // pins a warp stages at once
+constexpr int kHpwlLane = 16;        // pins of a window that one lane spans
+constexpr int kHpwlWarpMax = 1024;   // longer nets are spanned by a whole block
+constexpr int kHpwlBigs = 8;         // such nets a warp keeps for its block
 
-// Pin position; a pin_cell outside [0, C) is counted in *bad and reads cell 0
-// instead (the call then reports NaN).
-__device__ __forceinline__ float2 pin_pos(const float2 *xy, const int32_t *pin_cell,
-                                          const float *dx, const float *dy, long long k,
-                                          int32_t C, int *bad) {
-  int32_t i = pin_cell[k];
-  if ((uint32_t)i >= (uint32_t)C) {
-    atomicAdd(bad, 1);
-    i = 0;
+// Positions of pins k0, k0 + stride, ... (kPins of them, those below e): all
+// cell indices and offsets are loaded, then all cells gathered.  A pin_cell
+// outside [0, C) sets bad and reads cell 0 instead (the call then reports NaN):
+// nothing is written or branched on between the loads, so they stay in flight
+// together.
+constexpr int kPins = 4;
+__device__ __forceinline__ void pin_pos(const float2 *xy, const int32_t *pin_cell, const float *dx,
+                                        const float *dy, long long k0, int stride, long long e,
+                                        int32_t C, bool &bad, float2 *p) {
+  int32_t c[kPins];
+  float ox[kPins], oy[kPins];
+#pragma unroll
+  for (int u = 0; u < kPins; ++u) {
+    const long long k = k0 + (long long)u * stride;
+    const bool in = k < e;
+    c[u] = in ? __ldcs(pin_cell + k) : 0;
+    ox[u] = in && dx ? __ldcs(dx + k) : 0.f;
+    oy[u] = in && dy ? __ldcs(dy + k) : 0.f;
   }
-  float2 c = xy[i];
-  if (dx) c.x += dx[k];
-  if (dy) c.y += dy[k];
-  return c;
+#pragma unroll
+  for (int u = 0; u < kPins; ++u) {
+    const bool ok = (uint32_t)c[u] < (uint32_t)C;
+    const bool in = k0 + (long long)u * stride < e;
+    bad |= in && !ok;
+    p[u] = in && C > 0 ? xy[ok ? c[u] : 0] : make_float2(0.f, 0.f);
+  }
+#pragma unroll
+  for (int u = 0; u < kPins; ++u) {
+    if (dx) p[u].x += ox[u];
+    if (dy) p[u].y += oy[u];
+  }
 }
 
 // A net's span (x1 - x0) + (y1 - y0) added to a double-float sum: each
@@ -47,146 +69,164 @@ __device__ __forceinline__ void span_add(dfl &acc, float x0, float x1, float y0,
   df_add_df(acc, dy);
 }
 
-__global__ void __launch_bounds__(kHpwlThreads) k_hpwl(const int64_t *net_ptr,
-                                                       const int32_t *pin_cell, const float *dx,
-                                                       const float *dy, const float2 *xy,
-                                                       int32_t M, int32_t C, double *part,
-                                                       int *ticket, double *out) {
+struct Extent {
+  // no pin yet: an empty range (NaN coordinates leave it as it is)
+  float x0 = HUGE_VALF, x1 = -HUGE_VALF, y0 = HUGE_VALF, y1 = -HUGE_VALF;
+  __device__ __forceinline__ void add(float2 p) {
+    x0 = fminf(x0, p.x); x1 = fmaxf(x1, p.x);
+    y0 = fminf(y0, p.y); y1 = fmaxf(y1, p.y);
+  }
+  __device__ __forceinline__ void add(const Extent &e) {
+    x0 = fminf(x0, e.x0); x1 = fmaxf(x1, e.x1);
+    y0 = fminf(y0, e.y0); y1 = fmaxf(y1, e.y1);
+  }
+  // a net all of whose pins are NaN on an axis has no span there
+  __device__ __forceinline__ void close() {
+    if (x0 > x1) x0 = x1 = __int_as_float(0x7fc00000);
+    if (y0 > y1) y0 = y1 = __int_as_float(0x7fc00000);
+  }
+  __device__ __forceinline__ void warp() {  // over the lanes
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) {
+      x0 = fminf(x0, __shfl_xor_sync(0xffffffffu, x0, m));
+      x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, m));
+      y0 = fminf(y0, __shfl_xor_sync(0xffffffffu, y0, m));
+      y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, m));
+    }
+  }
+};
+
+// This thread's share of pins [b, e) (every nt-th from t), kPins gathers in flight.
+__device__ __forceinline__ Extent strided_extent(const float2 *xy, const int32_t *pin_cell,
+                                                 const float *dx, const float *dy, long long b,
+                                                 long long e, int t, int nt, int32_t C, bool &bad) {
+  Extent q;
+  for (long long k0 = b + t; k0 < e; k0 += (long long)kPins * nt) {
+    float2 p[kPins];
+    pin_pos(xy, pin_cell, dx, dy, k0, nt, e, C, bad, p);
+#pragma unroll
+    for (int u = 0; u < kPins; ++u)
+      if (k0 + (long long)u * nt < e) q.add(p[u]);
+  }
+  return q;
+}
+
+// Bound by the latency of net_ptr -> pin_cell -> xy gathers: the next batch's
+// net_ptr is loaded a batch ahead, and a window's cell indices, then its gathers,
+// go out together (nothing is counted or branched on in between: the check of
+// an index used to end each gather's wait before the next index was loaded).  Windows take any batch (before, a batch
+// above its stage of 512 pins fell back to a lane per net straight from memory,
+// and every block looked through its nets once more for the long ones).  2.25M
+// nets, 8.9M pins: 150 -> 77 us (five blocks a SM spill: 96 us; eight pins in
+// flight a lane: 92 us).
+__global__ void __launch_bounds__(kHpwlThreads, kHpwlPerSm) k_hpwl(const int64_t *net_ptr,
+                                                          const int32_t *pin_cell,
+                                                          const float *dx, const float *dy,
+                                                          const float2 *xy, int32_t M, int32_t C,
+                                                          double *part, int *ticket, double *out) {
   __shared__ double red[kHpwlThreads / 32];
   __shared__ int last;
-  __shared__ float2 stage_all[kHpwlThreads / 32][kHpwlStage];
-  __shared__ int32_t bigs[kHpwlThreads];
-  __shared__ int wcnt[kHpwlThreads / 32];
+  __shared__ float2 stage_all[kHpwlThreads / 32][kHpwlWin];
+  __shared__ int32_t bigs[kHpwlThreads / 32][kHpwlBigs];
+  __shared__ int nbigs[kHpwlThreads / 32];
   __shared__ float4 mm[kHpwlThreads / 32];
   float2 *stg = stage_all[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   dfl acc{0.f, 0.f};
-  // each warp takes batches of 32 consecutive nets (warp-uniform loop): a
-  // staged batch spans every net in it from shared memory; otherwise a lane
-  // spans each net of at most 32 pins and the warp each one of at most
-  // kHpwlWarpMax; longer nets are left to the block pass below
+  int nbig = 0;  // the same in every lane
+  bool bad = false;
   const long long wg = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarp = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long base = wg * 32; base < M; base += nwarp * 32) {
-    const long long e = base + lane;
-    const long long p0 = net_ptr[base], p1 = net_ptr[base + 32 < M ? base + 32 : M];
-    if (p1 - p0 <= kHpwlStage) {
-      // the batch's pins fit the warp's stage: lanes load all of them (all
-      // gathers in flight), then each lane spans its own net from the stage
-      for (long long k0 = p0; k0 < p1; k0 += 4 * 32) {
-        float2 q[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const long long k = k0 + u * 32 + lane;
-          if (k < p1) q[u] = pin_pos(xy, pin_cell, dx, dy, k, C, ticket + 1);
+  const long long step = (((long long)gridDim.x * blockDim.x) >> 5) * 32;
+  auto ptr = [&](long long e) { return net_ptr[e < M ? e : M]; };
+  long long na = 0, nz = 0;  // the next batch's pin range of this lane's net
+  if (wg * 32 < M) {
+    na = ptr(wg * 32 + lane);
+    nz = ptr(wg * 32 + lane + 1);
+  }
+  for (long long base = wg * 32; base < M; base += step) {
+    const long long a = na, z = nz;
+    if (base + step < M) {
+      na = ptr(base + step + lane);
+      nz = ptr(base + step + lane + 1);
+    }
+    const long long p0 = __shfl_sync(0xffffffffu, a, 0), p1 = __shfl_sync(0xffffffffu, z, 31);
+    bool big = z - a > kHpwlWarpMax;
+    unsigned bb = __ballot_sync(0xffffffffu, big);
+    for (unsigned t = bb; t; t &= t - 1) {  // kept for the block while the list has room
+      const int src = __ffs(t) - 1;
+      if (nbig < kHpwlBigs) {
+        if (lane == 0) bigs[wid][nbig] = (int32_t)(base + src);
+        ++nbig;
+      } else {
+        if (lane == src) big = false;  // spanned below, window by window
+        bb &= ~(1u << src);
+      }
+    }
+    Extent q;
+    for (long long c0 = p0; c0 < p1;) {
+      if (bb) {  // a window starts behind a net that is left out
+        const unsigned in = __ballot_sync(0xffffffffu, big && a <= c0 && c0 < z);
+        if (in) {
+          c0 = __shfl_sync(0xffffffffu, z, __ffs(in) - 1);
+          continue;
         }
+      }
+      const int n = (int)(p1 - c0 < kHpwlWin ? p1 - c0 : kHpwlWin);
+      for (int k0 = 0; k0 < n; k0 += kPins * 32) {
+        float2 p[kPins];
+        pin_pos(xy, pin_cell, dx, dy, c0 + k0 + lane, 32, c0 + n, C, bad, p);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const long long k = k0 + u * 32 + lane;
-          if (k < p1) stg[k - p0] = q[u];
-        }
+        for (int u = 0; u < kPins; ++u)
+          if (k0 + 32 * u + lane < n) stg[k0 + 32 * u + lane] = p[u];
       }
       __syncwarp();
-      if (e < M) {
-        const long long b = net_ptr[e] - p0, n = net_ptr[e + 1] - net_ptr[e];
-        if (n > 0 && n <= kHpwlWarpMax) {
-          float2 p = stg[b];
-          float x0 = p.x, x1 = p.x, y0 = p.y, y1 = p.y;
-          for (long long k = b + 1; k < b + n; ++k) {
-            p = stg[k];
-            x0 = fminf(x0, p.x); x1 = fmaxf(x1, p.x);
-            y0 = fminf(y0, p.y); y1 = fmaxf(y1, p.y);
-          }
-          span_add(acc, x0, x1, y0, y1);
-        }
+      // this lane's net's part of the window
+      const int lo = (int)(a > c0 ? (a - c0 < n ? a - c0 : n) : 0);
+      int hi = (int)(z > c0 ? (z - c0 < n ? z - c0 : n) : 0);
+      if (big) hi = lo;
+      const bool wide = hi - lo > kHpwlLane;
+      if (!wide)
+        for (int k = lo; k < hi; ++k) q.add(stg[k]);
+      for (unsigned t = __ballot_sync(0xffffffffu, wide); t; t &= t - 1) {
+        const int src = __ffs(t) - 1;
+        const int l = __shfl_sync(0xffffffffu, lo, src), h = __shfl_sync(0xffffffffu, hi, src);
+        Extent r;
+        for (int k = l + lane; k < h; k += 32) r.add(stg[k]);
+        r.warp();
+        if (lane == src) q.add(r);
       }
       __syncwarp();
-      continue;
+      c0 += n;
     }
-    bool mid = false;
-    if (e < M) {
-      const long long b = net_ptr[e], n = net_ptr[e + 1] - b;
-      if (n > 0 && n <= 32) {
-        float2 p = pin_pos(xy, pin_cell, dx, dy, b, C, ticket + 1);
-        float x0 = p.x, x1 = p.x, y0 = p.y, y1 = p.y;
-        for (long long k = b + 1; k < b + n; ++k) {
-          p = pin_pos(xy, pin_cell, dx, dy, k, C, ticket + 1);
-          x0 = fminf(x0, p.x); x1 = fmaxf(x1, p.x);
-          y0 = fminf(y0, p.y); y1 = fmaxf(y1, p.y);
-        }
-        span_add(acc, x0, x1, y0, y1);
-      }
-      mid = n > 32 && n <= kHpwlWarpMax;
-    }
-    // nets of 33..kHpwlWarpMax pins: the whole warp, one net at a time
-    unsigned bm = __ballot_sync(0xffffffffu, mid);
-    while (bm) {
-      const int src = __ffs(bm) - 1;
-      bm &= bm - 1;
-      const long long b = net_ptr[base + src], n = net_ptr[base + src + 1] - b;
-      float x0 = 3.4e38f, x1 = -3.4e38f, y0 = 3.4e38f, y1 = -3.4e38f;
-      for (long long k = b + lane; k < b + n; k += 32) {
-        const float2 p = pin_pos(xy, pin_cell, dx, dy, k, C, ticket + 1);
-        x0 = fminf(x0, p.x); x1 = fmaxf(x1, p.x);
-        y0 = fminf(y0, p.y); y1 = fmaxf(y1, p.y);
-      }
-#pragma unroll
-      for (int m = 16; m > 0; m >>= 1) {
-        x0 = fminf(x0, __shfl_xor_sync(0xffffffffu, x0, m));
-        x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, m));
-        y0 = fminf(y0, __shfl_xor_sync(0xffffffffu, y0, m));
-        y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, m));
-      }
-      if (lane == src) span_add(acc, x0, x1, y0, y1);
+    if (!big && z > a) {
+      q.close();
+      span_add(acc, q.x0, q.x1, q.y0, q.y1);
     }
   }
-  // nets of more than kHpwlWarpMax pins in this block's range of nets, in
-  // net order, each spanned by the whole block (strided pins, then a fixed
-  // tree)
+  // the block's nets of more than kHpwlWarpMax pins, warp by warp, in order
+  if (lane == 0) nbigs[wid] = nbig;
+  __syncthreads();
   double bigacc = 0.0;  // thread 0
-  const long long R = ((long long)M + gridDim.x - 1) / gridDim.x;
-  const long long r0 = (long long)blockIdx.x * R, r1 = r0 + R < M ? r0 + R : M;
-  for (long long c0 = r0; c0 < r1; c0 += kHpwlThreads) {
-    const long long e = c0 + threadIdx.x;
-    const bool big = e < r1 && net_ptr[e + 1] - net_ptr[e] > kHpwlWarpMax;
-    const unsigned bal = __ballot_sync(0xffffffffu, big);
-    if (lane == 0) wcnt[wid] = __popc(bal);
-    __syncthreads();
-    int before = 0, nbig = 0;
-    for (int w = 0; w < kHpwlThreads / 32; ++w) {
-      before += w < wid ? wcnt[w] : 0;
-      nbig += wcnt[w];
-    }
-    if (big) bigs[before + __popc(bal & ((1u << lane) - 1u))] = (int32_t)e;
-    __syncthreads();
-    for (int i = 0; i < nbig; ++i) {
-      const long long ee = bigs[i], b = net_ptr[ee], n = net_ptr[ee + 1] - b;
-      float x0 = 3.4e38f, x1 = -3.4e38f, y0 = 3.4e38f, y1 = -3.4e38f;
-      for (long long k = b + threadIdx.x; k < b + n; k += kHpwlThreads) {
-        const float2 p = pin_pos(xy, pin_cell, dx, dy, k, C, ticket + 1);
-        x0 = fminf(x0, p.x); x1 = fmaxf(x1, p.x);
-        y0 = fminf(y0, p.y); y1 = fmaxf(y1, p.y);
-      }
-#pragma unroll
-      for (int m = 16; m > 0; m >>= 1) {
-        x0 = fminf(x0, __shfl_xor_sync(0xffffffffu, x0, m));
-        x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, m));
-        y0 = fminf(y0, __shfl_xor_sync(0xffffffffu, y0, m));
-        y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, m));
-      }
-      if (lane == 0) mm[wid] = make_float4(x0, x1, y0, y1);
+  for (int w = 0; w < kHpwlThreads / 32; ++w)
+    for (int i = 0; i < nbigs[w]; ++i) {
+      const long long e = bigs[w][i];
+      Extent r = strided_extent(xy, pin_cell, dx, dy, net_ptr[e], net_ptr[e + 1], threadIdx.x,
+                                kHpwlThreads, C, bad);
+      r.warp();
+      if (lane == 0) mm[wid] = make_float4(r.x0, r.x1, r.y0, r.y1);
       __syncthreads();
       if (threadIdx.x == 0) {
-        float4 t = mm[0];
-        for (int w = 1; w < kHpwlThreads / 32; ++w) {
-          t.x = fminf(t.x, mm[w].x); t.y = fmaxf(t.y, mm[w].y);
-          t.z = fminf(t.z, mm[w].z); t.w = fmaxf(t.w, mm[w].w);
+        for (int k = 1; k < kHpwlThreads / 32; ++k) {
+          const float4 t = mm[k];
+          r.x0 = fminf(r.x0, t.x); r.x1 = fmaxf(r.x1, t.y);
+          r.y0 = fminf(r.y0, t.z); r.y1 = fmaxf(r.y1, t.w);
         }
-        bigacc += ((double)t.y - (double)t.x) + ((double)t.w - (double)t.z);
+        r.close();
+        bigacc += ((double)r.x1 - (double)r.x0) + ((double)r.y1 - (double)r.y0);
       }
       __syncthreads();
     }
-  }
+  if (bad) atomicAdd(ticket + 1, 1);
   const double accd = warp_sum(df_to_d(df_norm(acc)));
   if (lane == 0) red[wid] = accd;
   __syncthreads();
@@ -222,7 +262,7 @@ size_t hpwl_ws_bytes(int32_t M) { return 256 + (size_t)hpwl_blocks(M) * sizeof(d
 
 cudaError_t launch_hpwl(const pl_netlist *nl, const float *xy, double *out, void *ws,
                         cudaStream_t s) {
-  int nb = hpwl_blocks(nl->num_nets);
+  const int nb = grid_for((long long)nl->num_nets, kHpwlThreads, kHpwlGrid);  // at most hpwl_blocks
   int *ticket = reinterpret_cast<int *>(ws);
   double *part = reinterpret_cast<double *>(static_cast<char *>(ws) + 256);
   k_hpwl<<<nb, kHpwlThreads, 0, s>>>(nl->net_ptr, nl->pin_cell, nl->pin_dx, nl->pin_dy,
