@@ -15,6 +15,7 @@
 // midpoint, where the FP64 value is computed; for FP32 storage a double-float
 // value (about 2^-40) decides the rounding, except within its error bound of an
 // FP32 rounding midpoint.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -141,9 +142,8 @@ __device__ __forceinline__ float store_bits2(void *wbuf, uint64_t k, uint64_t k2
   return bf16_to_f(h);
 }
 
-// Cells are taken in tiles of kBinTile consecutive ids by the stable counting
+// Cells are taken in tiles of 2^tsh consecutive ids (hint_tile_shift) by the stable counting
 // sorts (bin buckets, macro lists).
-constexpr int kBinTile = 4096;
 constexpr int kMaxSmemBuckets = 12288;
 constexpr int kMacroSlots = 8;        // macros one cell may overlap in the tiled macro lists
 constexpr int kMaxSmemMacros = 12288;  // macros of the tiled macro lists (runs and masks in smem)
@@ -153,7 +153,7 @@ __global__ void k_hint_cells(HintGeo G, const float2 *xy, const uint8_t *ckind,
                              const uint8_t *hflag, const float *cw, const float *ch,
                              const int64_t *gptr, const uint32_t *glist, const float4 *ggeo,
                              int32_t *cell_bin, int32_t *n_ovl, int32_t *bcnt, int32_t *mcnt,
-                             int32_t *mtc, int ntile, int32_t *cmem, int *status) {
+                             int32_t *mtc, int ntile, int tsh, int32_t *cmem, int *status) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < G.C; i += gridDim.x * blockDim.x) {
     // the cell's inputs in flight together, before the kind test
     const uint8_t kd = ckind[i];
@@ -182,7 +182,7 @@ __global__ void k_hint_cells(HintGeo G, const float2 *xy, const uint8_t *ckind,
         if (overlaps(p.x, p.y, cwi, chi, mg.x, mg.y, mg.z, mg.w)) {
           const uint32_t m = glist[q];
           if (mtc) {
-            atomicAdd(&mtc[(long long)m * ntile + i / kBinTile], 1);
+            atomicAdd(&mtc[(long long)m * ntile + (i >> tsh)], 1);
             if (n < kMacroSlots) cmem[(long long)i * kMacroSlots + n] = (int32_t)m;
           } else {
             atomicAdd(&mcnt[m], 1);
@@ -217,7 +217,7 @@ __global__ void k_macro_scatter(HintGeo G, const float2 *xy, const uint8_t *ckin
   }
 }
 
-// Macro lists in ascending cell id without a sort: a CTA per tile of kBinTile
+// Macro lists in ascending cell id without a sort: a CTA per tile of 2^tsh
 // cells, counts per (macro, tile) macro-major and each cell's macros (at most
 // kMacroSlots) from k_hint_cells.  In rounds of blockDim cells the warps take
 // turns; inside a turn the lanes mark their macros in a per-macro lane mask,
@@ -225,16 +225,17 @@ __global__ void k_macro_scatter(HintGeo G, const float2 *xy, const uint8_t *ckin
 // turns), the macro's run so far and the number of lower lanes marked.
 __global__ void __launch_bounds__(256, 4) k_macro_tile_scatter(int32_t C, const int32_t *n_ovl,
                                                             const int32_t *cmem, int Mm,
-                                                            int ntile, const int64_t *off,
+                                                            int ntile, int tsh,
+                                                            const int64_t *off,
                                                             uint32_t *mlist) {
-  extern __shared__ uint32_t lmask[];  // [Mm] lane masks, then [Mm] runs (at most kBinTile)
+  extern __shared__ uint32_t lmask[];  // [Mm] lane masks, then [Mm] runs (at most 4096)
   uint16_t *run = reinterpret_cast<uint16_t *>(lmask + Mm);
   for (int k = threadIdx.x; k < Mm; k += blockDim.x) {
     run[k] = 0;
     lmask[k] = 0u;
   }
   __syncthreads();
-  const int t = blockIdx.x, i0 = t * kBinTile, i1 = min(C, i0 + kBinTile);
+  const int t = blockIdx.x, i0 = t << tsh, i1 = min(C, i0 + (1 << tsh));
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   // a round's cell memberships are loaded during the round before
@@ -293,21 +294,21 @@ __global__ void __launch_bounds__(256, 4) k_macro_tile_scatter(int32_t C, const 
 }
 
 // Bin buckets: key 2*bin + (baseWeight == 0).  A stable counting sort over
-// tiles of kBinTile consecutive cells writes every bucket in ascending cell id
+// tiles of 2^tsh consecutive cells writes every bucket in ascending cell id
 // directly (no sort).  Counts per (bucket, tile), bucket-major.
 
 __device__ __forceinline__ int bucket_of(const uint8_t *hflag, const int32_t *cell_bin, int i) {
   return 2 * cell_bin[i] + (hflag[i] ? 0 : 1);
 }
 
-__global__ void __launch_bounds__(256) k_bin_tile_count(int32_t C, int nbk, int ntile,
+__global__ void __launch_bounds__(256) k_bin_tile_count(int32_t C, int nbk, int ntile, int tsh,
                                                         const uint8_t *ckind,
                                                         const uint8_t *hflag,
                                                         const int32_t *cell_bin, int32_t *cnt) {
   extern __shared__ int32_t sc[];
   for (int k = threadIdx.x; k < nbk; k += blockDim.x) sc[k] = 0;
   __syncthreads();
-  const int t = blockIdx.x, i0 = t * kBinTile, i1 = min(C, i0 + kBinTile);
+  const int t = blockIdx.x, i0 = t << tsh, i1 = min(C, i0 + (1 << tsh));
   for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x)
     if (ckind[i] == 0) atomicAdd(&sc[bucket_of(hflag, cell_bin, i)], 1);
   __syncthreads();
@@ -316,7 +317,7 @@ __global__ void __launch_bounds__(256) k_bin_tile_count(int32_t C, int nbk, int 
 
 // Rounds of blockDim cells; inside a round the warps take turns (so equal
 // buckets keep cell order), lanes of a warp rank themselves with match_any.
-__global__ void __launch_bounds__(256) k_bin_tile_scatter(int32_t C, int nbk, int ntile,
+__global__ void __launch_bounds__(256) k_bin_tile_scatter(int32_t C, int nbk, int ntile, int tsh,
                                                           const uint8_t *ckind,
                                                           const uint8_t *hflag,
                                                           const int32_t *cell_bin,
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(256) k_bin_tile_scatter(int32_t C, int nbk, in
   extern __shared__ int32_t run[];
   for (int k = threadIdx.x; k < nbk; k += blockDim.x) run[k] = 0;
   __syncthreads();
-  const int t = blockIdx.x, i0 = t * kBinTile, i1 = min(C, i0 + kBinTile);
+  const int t = blockIdx.x, i0 = t << tsh, i1 = min(C, i0 + (1 << tsh));
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   for (int base = i0; base < i1; base += blockDim.x) {
@@ -357,7 +358,7 @@ __global__ void __launch_bounds__(256) k_bin_tile_scatter(int32_t C, int nbk, in
 // barrier a cell's place is the key's run so far, plus the same key's cells in
 // the round's lower warps, plus its lower lanes of the same key, which is its
 // place in cell order.  Two barriers per round instead of one per warp.
-__global__ void __launch_bounds__(256) k_bin_tile_scatter_wc(int32_t C, int nbk, int ntile,
+__global__ void __launch_bounds__(256) k_bin_tile_scatter_wc(int32_t C, int nbk, int ntile, int tsh,
                                                              const uint8_t *ckind,
                                                              const uint8_t *hflag,
                                                              const int32_t *cell_bin,
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(256) k_bin_tile_scatter_wc(int32_t C, int nbk,
   for (int k = threadIdx.x; k < nbk; k += blockDim.x) run[k] = 0;
   for (int k = threadIdx.x; k < 8 * nbk; k += blockDim.x) wc[k] = 0;
   __syncthreads();
-  const int t = blockIdx.x, i0 = t * kBinTile, i1 = min(C, i0 + kBinTile);
+  const int t = blockIdx.x, i0 = t << tsh, i1 = min(C, i0 + (1 << tsh));
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   for (int base = i0; base < i1; base += blockDim.x) {
@@ -1665,7 +1666,14 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   TRY(ensure(g->bcnt, (size_t)(nbk + 1) * 4));
   TRY(ensure(g->mcnt, (size_t)(Mm + 1) * 4));
   if (!tiled) TRY(cudaMemsetAsync(g->bcnt.p, 0, (size_t)(nbk + 1) * 4, s));
-  const int ntile = (int)((C + kBinTile - 1) / kBinTile) > 0 ? (int)((C + kBinTile - 1) / kBinTile) : 1;
+  int tsh = hint_tile_shift(C, NB, Mm);
+  {
+    // (the counts of a workspace with little room left: the largest tiles)
+    const Arena *ar = current_arena();
+    const uint64_t nt = std::max<uint64_t>(1, ((uint64_t)C + (1u << tsh) - 1) >> tsh);
+    if ((nt * ((uint64_t)Mm + 2 * (uint64_t)NB)) * 12 > (ar->cap - ar->used) / 4) tsh = 12;
+  }
+  const int ntile = std::max(1, (int)(((int64_t)C + (1 << tsh) - 1) >> tsh));
   // macro lists by a tiled counting sort when the macros' run counters fit
   // shared memory (else: scatter by atomics, then a segmented sort)
   const bool tiledm = Mm > 0 && Mm <= kMaxSmemMacros;
@@ -1681,7 +1689,7 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
       G, xy, P<uint8_t>(g->ckind), P<uint8_t>(g->hflag), P<float>(g->cw), P<float>(g->ch),
       P<int64_t>(g->gptr), P<uint32_t>(g->glist), P<float4>(g->ggeo), P<int32_t>(g->cell_bin),
       P<int32_t>(g->n_ovl), tiled ? nullptr : P<int32_t>(g->bcnt), P<int32_t>(g->mcnt),
-      tiledm ? P<int32_t>(g->mtc) : nullptr, ntile, tiledm ? P<int32_t>(g->cmem) : nullptr,
+      tiledm ? P<int32_t>(g->mtc) : nullptr, ntile, tsh, tiledm ? P<int32_t>(g->cmem) : nullptr,
       status);
   note_launch();
   // H2: bucket offsets
@@ -1708,7 +1716,7 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
     stmp = g->tmp[7].p;
     cm = P<int32_t>(g->tmp[5]);
     cmo = P<int64_t>(g->tmp[6]);
-    k_bin_tile_count<<<ntile, 256, (size_t)nbk * 4, s>>>(C, nbk, ntile, P<uint8_t>(g->ckind),
+    k_bin_tile_count<<<ntile, 256, (size_t)nbk * 4, s>>>(C, nbk, ntile, tsh, P<uint8_t>(g->ckind),
                                                         P<uint8_t>(g->hflag),
                                                         P<int32_t>(g->cell_bin), cm);
     note_launch();
@@ -1740,10 +1748,10 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   if (tiled) {
     if ((size_t)nbk * 20 <= 48 * 1024)
       k_bin_tile_scatter_wc<<<ntile, 256, (size_t)nbk * 20, s>>>(
-          C, nbk, ntile, P<uint8_t>(g->ckind), P<uint8_t>(g->hflag), P<int32_t>(g->cell_bin), cmo,
+          C, nbk, ntile, tsh, P<uint8_t>(g->ckind), P<uint8_t>(g->hflag), P<int32_t>(g->cell_bin), cmo,
           P<uint32_t>(g->blist));
     else
-      k_bin_tile_scatter<<<ntile, 256, (size_t)nbk * 4, s>>>(C, nbk, ntile, P<uint8_t>(g->ckind),
+      k_bin_tile_scatter<<<ntile, 256, (size_t)nbk * 4, s>>>(C, nbk, ntile, tsh, P<uint8_t>(g->ckind),
                                                             P<uint8_t>(g->hflag),
                                                             P<int32_t>(g->cell_bin), cmo,
                                                             P<uint32_t>(g->blist));
@@ -1793,7 +1801,7 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
                            kMaxSmemMacros * 6);
     });
     k_macro_tile_scatter<<<ntile, 256, (size_t)Mm * 6, s3>>>(C, P<int32_t>(g->n_ovl),
-                                                            P<int32_t>(g->cmem), Mm, ntile,
+                                                            P<int32_t>(g->cmem), Mm, ntile, tsh,
                                                             P<int64_t>(g->mtoff),
                                                             P<uint32_t>(g->mlist));
     note_launch();

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 
 #include "../../include/pl.h"
@@ -186,6 +187,22 @@ void for_each_buf(pl_graph *g, int kind, F f) {
                  &g->xa, &g->xb, &g->xc, &g->g0, &g->ua, &g->ub, &g->acc, &g->gsc, &g->q4a,
                  &g->q4b, &g->status, &g->stage, &g->star_w, &g->lscr};
   for (Buf *b : rest) f(*b);
+}
+
+// Cells per tile of the hint build's counting sorts, as a shift: a CTA places a
+// tile's cells in rounds of 256, one after the other, so tiles as small as keep
+// their number (two per SM) and the count tables small.  (Hint build of 20k
+// cells, 64 x 64 bins: bucket lists 43 -> 8 us, macro lists 64 -> 10 us with
+// tiles of 512 instead of 4096.)
+constexpr int64_t kTileCounts = 1500000;  // words of a count table, except with the largest tiles
+inline int hint_tile_shift(int64_t cells, int64_t bins, int64_t macros) {
+  int sh = 9;
+  while (sh < 12) {
+    const int64_t n = (cells + (1 << sh) - 1) >> sh;
+    if (n <= 304 && n * std::max(2 * bins, macros) <= kTileCounts) break;
+    ++sh;
+  }
+  return sh;
 }
 
 void set_error(const char *fmt, ...);

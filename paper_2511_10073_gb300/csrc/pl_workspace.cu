@@ -121,8 +121,10 @@ double workspace_bound(const pl_netlist *nl, const pl_params *p) {
   // one hint build
   Plan h;
   const double nmov = C, nml = nmov * kMaxCellMacros, nbk = 2 * NB;
-  const double ntile = std::max(1.0, std::ceil(C / 4096.0));
-  const double nmt = Mm * ntile, ncm = nbk * ntile;
+  // counts per tile: tables of at most kTileCounts words, or the largest tiles'
+  const double nt12 = std::max(1.0, std::ceil(C / 4096.0)), nt9 = std::max(1.0, std::ceil(C / 512.0));
+  auto counts = [&](double keys) { return std::max(std::min((double)kTileCounts, keys * nt9), keys * nt12); };
+  const double nmt = counts(Mm), ncm = counts(nbk);
   h.add(scan_b(N + 1));
   h.add(C * 4 + 16);
   h.add(C * 4 + 16);
