@@ -265,7 +265,7 @@ __device__ __forceinline__ void chunk_piece(const int32_t *colp, const void *wp,
 #pragma unroll
     for (int q = 0; q < kChunkBatch; ++q) {
       const uint64_t k = k0 + q * 32 + lane;
-      xv[q] = k < e ? __ldg(x + (size_t)cc[q] * xs) : make_float2(0.f, 0.f);
+      xv[q] = k < e ? __ldca(x + (size_t)cc[q] * xs) : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int q = 0; q < kChunkBatch; ++q) {
@@ -337,7 +337,7 @@ __device__ __forceinline__ void row_piece(const int32_t *col, const void *w, uin
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (c[u] >= 0) {
-        const float2 xv = __ldg(x + c[u]);
+        const float2 xv = __ldca(x + c[u]);
         sx = fmaf(wv[u], xv.x, sx);
         sy = fmaf(wv[u], xv.y, sy);
       }
@@ -378,7 +378,7 @@ __device__ __forceinline__ void slot_piece(const StepArgs &A, long long v, int h
 #pragma unroll
     for (int u = 0; u < kSlotUnroll; ++u) {
       if (cb[u] >= 0) {
-        const float2 xv = __ldg(xb + cb[u]);
+        const float2 xv = __ldca(xb + cb[u]);
         sx = fmaf(wv[u], xv.x, sx);
         sy = fmaf(wv[u], xv.y, sy);
       }
@@ -412,7 +412,7 @@ __device__ __forceinline__ void slot_piece_fast(const StepArgs &A, long long v, 
 #pragma unroll
   for (int u = 0; u < kSlotUnroll; ++u) {
     if (cb[u] >= 0) {
-      const float2 xv = __ldg(xb + cb[u]);
+      const float2 xv = __ldca(xb + cb[u]);
       sx = fmaf(wv[u], xv.x, sx);
       sy = fmaf(wv[u], xv.y, sy);
     }
@@ -461,7 +461,7 @@ __device__ __forceinline__ void row_groups(const int32_t *col, const void *w, ui
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const bool in = gg + q >= k && gg + q < e;
-        xv[q] = in ? __ldg(x + ci[q]) : make_float2(0.f, 0.f);
+        xv[q] = in ? __ldca(x + ci[q]) : make_float2(0.f, 0.f);
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -669,6 +669,44 @@ __global__ void __launch_bounds__(kHubRows * 32) k_hub_rows(StepArgs A) {
   hub_rows_block<WT, MODE>(A, blockIdx.x, sums);
 }
 
+// One power of the refinement filter in two launches, for designs whose units
+// do not fill the chip: hub chunks, bin chunks and short-row groups are
+// independent of one another and go in one launch, a warp per unit, the longer
+// units first; the hub rows follow.  Both launches are programmatic dependents
+// of the one before: their blocks are placed while it runs and wait for its
+// completion before they touch memory.  A launch lets its own dependents in only
+// after that wait, so no more than one launch is ever ahead, and x is read with
+// coherent loads (it is written while a waiting launch already exists).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+template <int WT, bool NINE>
+__global__ void __launch_bounds__(256, 4) k_power_units(StepArgs A, long long nbin) {
+  pdl_wait();
+  pdl_release();
+  long long u = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (u < A.nchunks) {
+    warp_chunk<WT, MODE_HR>(A, (int)u);
+    return;
+  }
+  u -= A.nchunks;
+  if (u < nbin) {
+    if (u < A.bchunk[A.B.NB])
+      bin_chunk<WT, false, NINE>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, u);
+    return;
+  }
+  u -= nbin;
+  if (u * (32 / kRowLanes) < A.nrows) rows_group<WT, MODE_HR>(A, u * (32 / kRowLanes));
+}
+
+template <int WT>
+__global__ void __launch_bounds__(kHubRows * 32) k_power_hubs(StepArgs A) {
+  __shared__ float4 sums[kHubRows];
+  pdl_wait();
+  pdl_release();
+  hub_rows_block<WT, MODE_HR>(A, blockIdx.x, sums);
+}
+
 // ------------------------------------------------------------- helpers
 __global__ void k_init_signal(int64_t N, int32_t C, uint64_t seed, const float2 *xy0,
                               const uint8_t *nkind, const float2 *fixedp, double xl, double yl,
@@ -853,10 +891,52 @@ static int graph_nsm(pl_graph *g) {
   return g->nsm;
 }
 
+// Launches kernel k as a programmatic dependent of the launch before it on s.
+template <typename... P, typename... Q>
+static cudaError_t launch_pdl(void (*k)(P...), int grid, int block, cudaStream_t s, Q... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)block);
+  c.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
+// Blocks of k_power_units per SM up to which a refinement product takes that
+// form.  Above, the short rows' own kernel (40 registers, one persistent wave)
+// beside the hub and bin kernels on the second stream is the better one.  A round
+// (hint build and eight powers): 20k cells on 64 x 64 bins 549 -> 506 us, 210k
+// cells 558 -> 531 us, a whole initializer of 2k cells 1557 -> 1331 us; 1.1M cells
+// (two powers) 763 us on two streams, 787 us this way; 2.2M cells 2257 and 2651 us.
+constexpr long long kPowerBlocksPerSm = 16;
+
 template <int MODE>
 static cudaError_t launch_step(const StepArgs &A, double bytes, int wdtype, cudaStream_t s,
                                pl_graph *g) {
   const int nsm = graph_nsm(g);
+  if (MODE == MODE_HR && A.nlong > 0 && A.bpart) {
+    const long long nbin = g->nbc_max, rg = 32 / kRowLanes;
+    const long long blocks = ((long long)A.nchunks + nbin + (A.nrows + rg - 1) / rg + 7) / 8;
+    if (blocks <= kPowerBlocksPerSm * nsm) {
+      const bool prof = prof_on();
+      if (prof) prof_begin(s, PROF_HR, bytes);
+      const bool bf = wdtype == PL_W_BF16, nine = A.B.W == 9;
+      auto ku = bf ? (nine ? k_power_units<1, true> : k_power_units<1, false>)
+                   : (nine ? k_power_units<0, true> : k_power_units<0, false>);
+      cudaError_t e = launch_pdl(ku, (int)blocks, 256, s, A, nbin);
+      if (e == cudaSuccess)
+        e = launch_pdl(bf ? k_power_hubs<1> : k_power_hubs<0>, (A.nlong + kHubRows - 1) / kHubRows,
+                       kHubRows * 32, s, A);
+      note_launch();
+      note_launch();
+      if (prof) prof_end(s);
+      return e != cudaSuccess ? e : cudaGetLastError();
+    }
+  }
   // short rows: one wave of resident blocks, row groups dealt round robin
   int *occ = g->occ_rows[MODE];
   const int wi = wdtype == PL_W_BF16 ? 1 : 0;
@@ -868,7 +948,7 @@ static cudaError_t launch_step(const StepArgs &A, double bytes, int wdtype, cuda
   }
   const bool prof = prof_on();
   if (prof) prof_begin(s, MODE == MODE_HR ? PROF_HR : PROF_GIFT, bytes);
-  const bool fork = A.nchunks > 0;
+  const bool fork = A.nlong > 0;
   if (fork) {
     cudaError_t e = ensure_side(g);
     if (e == cudaSuccess) e = cudaEventRecord(g->ev_fork, s);
@@ -877,9 +957,11 @@ static cudaError_t launch_step(const StepArgs &A, double bytes, int wdtype, cuda
     cudaStream_t sh = g->side;
     const long long want = ((long long)A.nchunks + 7) / 8;
     const int hgrid = (int)(want < 8LL * nsm ? want : 8LL * nsm);
-    if (wi) k_spmm_hub<1, MODE><<<hgrid, 256, 0, sh>>>(A);
-    else k_spmm_hub<0, MODE><<<hgrid, 256, 0, sh>>>(A);
-    note_launch();
+    if (hgrid) {
+      if (wi) k_spmm_hub<1, MODE><<<hgrid, 256, 0, sh>>>(A);
+      else k_spmm_hub<0, MODE><<<hgrid, 256, 0, sh>>>(A);
+      note_launch();
+    }
     if (MODE == MODE_HR && A.bpart) {
       // bin rows: chunk partials of the window blocks times the cells' x
       const long long bwant = (g->nbc_max + kBinThreads / 32 - 1) / (kBinThreads / 32);
@@ -938,7 +1020,7 @@ static cudaError_t launch_pair(const StepArgs &A, double bytes, int wdtype, cuda
   }
   const bool prof = prof_on();
   if (prof) prof_begin(s, PROF_GIFT, bytes);
-  const bool fork = A.nchunks > 0;
+  const bool fork = A.nlong > 0;
   if (fork) {
     cudaError_t e = ensure_side(g);
     if (e == cudaSuccess) e = cudaEventRecord(g->ev_fork, s);

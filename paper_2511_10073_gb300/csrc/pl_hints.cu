@@ -594,7 +594,7 @@ __device__ __forceinline__ RowLen row_len(const LayIn &A, long long v) {
   return r;
 }
 __device__ __forceinline__ uint32_t row_chunks(uint64_t cl) {
-  return cl == 0 ? 1u : (uint32_t)((cl + kChunk - 1) / kChunk);
+  return (uint32_t)((cl + kChunk - 1) / kChunk);  // none for a row without stored entries (bin rows)
 }
 
 constexpr int kLayPer = 8;                 // rows per lane (a warp: 256 consecutive rows)
