@@ -525,10 +525,15 @@ __device__ __forceinline__ void rows_group(const StepArgs &A, long long base) {
 
 template <int WT, int MODE>
 __global__ void __launch_bounds__(kRowThreads, 6) k_spmm_rows(StepArgs A) {
-  constexpr int RPW = 32 / kRowLanes;
-  const long long gw = ((long long)blockIdx.x * kRowThreads + threadIdx.x) >> 5;
-  const long long nw = ((long long)gridDim.x * kRowThreads) >> 5;
-  for (long long base = gw * RPW; base < A.nrows; base += nw * RPW) rows_group<WT, MODE>(A, base);
+  constexpr int RPW = 32 / kRowLanes, WPB = kRowThreads / 32;
+  const int wid = threadIdx.x >> 5;
+  // cells: a run of consecutive row groups per block
+  const long long nc = A.C / RPW, per = (nc + gridDim.x - 1) / gridDim.x;
+  const long long c0 = blockIdx.x * per, c1 = c0 + per < nc ? c0 + per : nc;
+  for (long long k = c0 + wid; k < c1; k += WPB) rows_group<WT, MODE>(A, k * RPW);
+  // the other rows (macro pins, stars: very uneven) dealt in turn
+  const long long gw = (long long)blockIdx.x * WPB + wid, nw = (long long)gridDim.x * WPB;
+  for (long long base = (nc + gw) * RPW; base < A.nrows; base += nw * RPW) rows_group<WT, MODE>(A, base);
 }
 
 // A GiFt chain pair over the short rows of the static matrix: the same
@@ -1140,6 +1145,7 @@ pl_status run_gift(pl_graph *g, const pl_params *p, const float *in, float *out,
   float *ga2 = gq + N, *gb2 = ga2 + N, *gq2 = gb2 + N;
   StepArgs A{};
   fill_matrix(A, g->st, nullptr);
+  A.C = g->C;
   const double bytes = spmm_bytes((double)(g->st.nnz_s + g->st.nnz_l), (double)N, g->wdtype);
   fill_nodes(A, g);
   A.acc = P<double2>(g->acc);
