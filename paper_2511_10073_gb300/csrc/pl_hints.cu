@@ -1921,6 +1921,8 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
         P<int32_t>(m.lchunk), P<int64_t>(g->moff), P<uint32_t>(g->mlist), P<int32_t>(g->n_ovl),
         P<uint64_t>(g->mac_base), P<int32_t>(m.col), m.w.p, cpart);
     note_launch();
+  }
+  if (nl_max) {
     k_hub_finalize<<<grid_for((long long)nl_max * 32, 256), 256, 0, s>>>(
         G, B, &tot->f, P<int32_t>(m.lrow), P<int32_t>(m.lchunk), cpart, P<int32_t>(g->bchunk),
         P<float4>(g->bdeg),
