@@ -143,6 +143,55 @@ __global__ void k_scan_apply(const Tin *in, Tout *out, long long n, const Tout *
   if (threadIdx.x == 0 && base + SCAN_B >= n) out[n] = off + tot;
 }
 
+// A scan of up to kScanOne values by one block, SCAN_ONE_B at a time: one launch
+// instead of three.
+constexpr int SCAN_ONE_T = 1024, SCAN_ONE_V = 8, SCAN_ONE_B = SCAN_ONE_T * SCAN_ONE_V;
+constexpr long long kScanOne = 4 * SCAN_ONE_B;
+template <typename Tin, typename Tout>
+__global__ void __launch_bounds__(SCAN_ONE_T) k_scan_one(const Tin *in, Tout *out, int n) {
+  __shared__ Tout wsum[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  Tout carry = 0;
+  for (int b0 = 0; b0 < n; b0 += SCAN_ONE_B) {
+    // warp w holds 256 consecutive values, value 32 k + lane of them in v[k]
+    const int i0 = b0 + w * 32 * SCAN_ONE_V + lane;
+    Tout v[SCAN_ONE_V], x[SCAN_ONE_V], tot = 0;
+#pragma unroll
+    for (int k = 0; k < SCAN_ONE_V; ++k) v[k] = i0 + 32 * k < n ? (Tout)in[i0 + 32 * k] : Tout(0);
+#pragma unroll
+    for (int k = 0; k < SCAN_ONE_V; ++k) {
+      x[k] = v[k];
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const Tout y = __shfl_up_sync(0xffffffffu, x[k], d);
+        if (lane >= d) x[k] += y;
+      }
+      const Tout t = __shfl_sync(0xffffffffu, x[k], 31);
+      x[k] += tot - v[k];
+      tot += t;
+    }
+    if (lane == 0) wsum[w] = tot;
+    __syncthreads();
+    if (w == 0) {
+      Tout t = wsum[lane];
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const Tout y = __shfl_up_sync(0xffffffffu, t, d);
+        if (lane >= d) t += y;
+      }
+      wsum[lane] = t;
+    }
+    __syncthreads();
+    const Tout off = carry + (w ? wsum[w - 1] : Tout(0));
+#pragma unroll
+    for (int k = 0; k < SCAN_ONE_V; ++k)
+      if (i0 + 32 * k < n) out[i0 + 32 * k] = off + x[k];
+    carry += wsum[31];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) out[n] = carry;
+}
+
 size_t scan_tmp_bytes(long long n) {
   size_t b = 0;
   while (n > SCAN_B) {
@@ -159,8 +208,8 @@ cudaError_t exclusive_scan(const Tin *in, Tout *out, long long n, void *tmp, cud
     return cudaMemsetAsync(out, 0, sizeof(Tout), s);
   }
   long long nb = (n + SCAN_B - 1) / SCAN_B;
-  if (nb == 1) {
-    k_scan_apply<Tin, Tout><<<1, SCAN_T, 0, s>>>(in, out, n, nullptr);
+  if (n <= kScanOne) {
+    k_scan_one<Tin, Tout><<<1, SCAN_ONE_T, 0, s>>>(in, out, (int)n);
     note_launch();
     return cudaGetLastError();
   }
@@ -312,10 +361,9 @@ __device__ __forceinline__ void warp_bitonic_regs(K (&key)[R], int lane) {
 
 // Groups of W lanes (W = 8, 16, 32) each sort one segment of at most W keys.
 template <typename K, int MODE, int W>
-__global__ void __launch_bounds__(256) k_seg_group(K *keys, const int64_t *off, int32_t *cnt,
-                                                   int32_t *mcol, int64_t *mval,
-                                                   const int32_t *list, const SegLists *ln,
-                                                   int cls) {
+__device__ __forceinline__ void seg_group(K *keys, const int64_t *off, int32_t *cnt, int32_t *mcol,
+                                          int64_t *mval, const int32_t *list, const SegLists *ln,
+                                          int cls) {
   const int lane = threadIdx.x & 31, sub = lane & (W - 1);
   const unsigned gmask = (W == 32) ? 0xffffffffu : (((1u << W) - 1u) << (lane & ~(W - 1)));
   const unsigned lt = (1u << lane) - 1u;
@@ -381,13 +429,11 @@ __global__ void __launch_bounds__(256) k_seg_group(K *keys, const int64_t *off, 
 // through the warp's shared-memory slice for the compaction (each lane a
 // contiguous run of R positions).
 template <typename K, int MODE, int R>
-__global__ void __launch_bounds__(256) k_seg_regs(K *keys, const int64_t *off, int32_t *cnt,
-                                                  int32_t *mcol, int64_t *mval,
-                                                  const int32_t *list, const SegLists *ln,
-                                                  int cls) {
-  __shared__ K sk[8][32 * R];
+__device__ __forceinline__ void seg_regs(K *keys, const int64_t *off, int32_t *cnt, int32_t *mcol,
+                                         int64_t *mval, const int32_t *list, const SegLists *ln,
+                                         int cls, K *sk) {
   const int lane = threadIdx.x & 31;
-  K *a = sk[threadIdx.x >> 5];
+  K *a = sk + (threadIdx.x >> 5) * (32 * R);
   const int nl = ln->n[cls];
   for (long long it = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; it < nl;
        it += ((long long)gridDim.x * blockDim.x) >> 5) {
@@ -493,11 +539,9 @@ __device__ void cta_compact(K *a, long long n, long long o, long long s, int32_t
 }
 
 template <typename K, int MODE>
-__global__ void __launch_bounds__(SEG_T) k_seg_cta(K *keys, const int64_t *off, int32_t *cnt,
-                                                   int32_t *mcol, int64_t *mval,
-                                                   const int32_t *med, const SegLists *lists) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  K *a = reinterpret_cast<K *>(smraw);
+__device__ __forceinline__ void seg_cta(K *keys, const int64_t *off, int32_t *cnt, int32_t *mcol,
+                                        int64_t *mval, const int32_t *med, const SegLists *lists,
+                                        K *a) {
   const int nmed = lists->n[7];
   for (int it = blockIdx.x; it < nmed; it += gridDim.x) {
     long long s = med[it];
@@ -515,6 +559,34 @@ __global__ void __launch_bounds__(SEG_T) k_seg_cta(K *keys, const int64_t *off, 
       cta_compact<K, MODE>(a, n, o, s, cnt, mcol, mval, keys);
     }
   }
+}
+
+// All size classes in one launch, longest segments first; every block takes its
+// share of each class.  (As a launch per class, the long classes' latency and
+// eight launches followed one another.  GSP start of 210k cells: 874 us with
+// separate launches, 783 us with one; whole initializer: 2k cells 1282 and
+// 1202 us, 2.2M cells 9.67 ms either way, although 64 registers leave the short
+// classes half the warps.)
+template <typename K, int MODE>
+__global__ void __launch_bounds__(SEG_T, 4) k_seg_all(K *keys, const int64_t *off, int32_t *cnt,
+                                                      int32_t *mcol, int64_t *mval,
+                                                      const int32_t *cl, long long nseg,
+                                                      const SegLists *lists) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  K *a = reinterpret_cast<K *>(smraw);  // SEG_CAP keys: one CTA's segment, or 8 warps' 512
+  static_assert(SEG_T == 256 && SEG_CAP >= 8 * 32 * 16, "the warps' slices share the CTA's stage");
+  seg_cta<K, MODE>(keys, off, cnt, mcol, mval, cl + 7 * nseg, lists, a);
+  __syncthreads();
+  seg_regs<K, MODE, 16>(keys, off, cnt, mcol, mval, cl + 6 * nseg, lists, 6, a);
+  __syncthreads();  // the next class' slices lie elsewhere in the stage
+  seg_regs<K, MODE, 8>(keys, off, cnt, mcol, mval, cl + 5 * nseg, lists, 5, a);
+  __syncthreads();
+  seg_regs<K, MODE, 4>(keys, off, cnt, mcol, mval, cl + 4 * nseg, lists, 4, a);
+  __syncthreads();
+  seg_regs<K, MODE, 2>(keys, off, cnt, mcol, mval, cl + 3 * nseg, lists, 3, a);
+  seg_group<K, MODE, 32>(keys, off, cnt, mcol, mval, cl + 2 * nseg, lists, 2);
+  seg_group<K, MODE, 16>(keys, off, cnt, mcol, mval, cl + nseg, lists, 1);
+  seg_group<K, MODE, 8>(keys, off, cnt, mcol, mval, cl, lists, 0);
 }
 
 // Segments longer than SEG_CAP, spread over all CTAs: each is cut into units
@@ -694,24 +766,15 @@ cudaError_t segmented_sort(K *keys, const int64_t *off, long long nseg, long lon
   k_seg_classify<K, MODE><<<grid_for(nseg, 256), 256, 0, s>>>(keys, off, nseg, cnt, mcol, mval,
                                                               cl, lists);
   note_launch();
-  // every class kernel reads its list length on the device (no host round
-  // trip); an empty class costs one launch that returns at once
-  const int gb = 152 * 8;
-  k_seg_group<K, MODE, 8><<<gb, 256, 0, s>>>(keys, off, cnt, mcol, mval, cl, lists, 0);
-  k_seg_group<K, MODE, 16><<<gb, 256, 0, s>>>(keys, off, cnt, mcol, mval, cl + nseg, lists, 1);
-  k_seg_group<K, MODE, 32><<<gb, 256, 0, s>>>(keys, off, cnt, mcol, mval, cl + 2 * nseg, lists, 2);
-  k_seg_regs<K, MODE, 2><<<gb, 256, 0, s>>>(keys, off, cnt, mcol, mval, cl + 3 * nseg, lists, 3);
-  k_seg_regs<K, MODE, 4><<<gb, 256, 0, s>>>(keys, off, cnt, mcol, mval, cl + 4 * nseg, lists, 4);
-  k_seg_regs<K, MODE, 8><<<gb, 256, 0, s>>>(keys, off, cnt, mcol, mval, cl + 5 * nseg, lists, 5);
-  k_seg_regs<K, MODE, 16><<<gb, 256, 0, s>>>(keys, off, cnt, mcol, mval, cl + 6 * nseg, lists, 6);
-  for (int q = 0; q < 7; ++q) note_launch();
-  size_t sm = SEG_CAP * sizeof(K);
+  const size_t sm = SEG_CAP * sizeof(K);
   static std::once_flag attr_once;
   std::call_once(attr_once, [sm] {
-    cudaFuncSetAttribute(k_seg_cta<K, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_seg_all<K, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaFuncSetAttribute(k_big_units<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   });
-  k_seg_cta<K, MODE><<<152 * 4, SEG_T, sm, s>>>(keys, off, cnt, mcol, mval, cl + 7 * nseg, lists);
+  // every class reads its list length on the device (no host round trip)
+  k_seg_all<K, MODE><<<grid_for(nseg, 64, 152 * 4), SEG_T, sm, s>>>(keys, off, cnt, mcol, mval, cl, nseg,
+                                                                   lists);
   note_launch();
   if (nkeys > SEG_CAP && (maxlen < 0 || maxlen > SEG_CAP)) {
     // The unit prefix overwrites the lists of the small classes (consumed by
