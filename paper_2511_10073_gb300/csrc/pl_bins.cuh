@@ -230,7 +230,45 @@ __device__ __forceinline__ void bin_row_chunks(const BinGeo &B, int b, const int
   *e = warp_sum_df(se);
 }
 
-// Chunks of each bin's hint bucket: counts, to be scanned into bchunk.
+// First chunk of each bin's hint bucket and the bucket of each chunk, by one
+// block (a thread per bin, 1024 at a time, writes its bucket's chunks).
+constexpr int kBinsOneBlock = 16384;
+static __global__ void __launch_bounds__(1024) k_bin_chunks(int NB, const int64_t *boff,
+                                                            int32_t *bchunk, int32_t *cown) {
+  __shared__ int ws[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int carry = 0;
+  for (int b0 = 0; b0 < NB; b0 += 1024) {
+    const int b = b0 + (int)threadIdx.x;
+    const int n = b < NB ? (int)((boff[2 * b + 1] - boff[2 * b] + kBinChunk - 1) / kBinChunk) : 0;
+    int x = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, d);
+      if (lane >= d) x += y;
+    }
+    if (lane == 31) ws[w] = x;
+    __syncthreads();
+    if (w == 0) {
+      int t = ws[lane];
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, t, d);
+        if (lane >= d) t += y;
+      }
+      ws[lane] = t;
+    }
+    __syncthreads();
+    const int c0 = carry + (w ? ws[w - 1] : 0) + x - n;
+    if (b < NB) bchunk[b] = c0;
+    for (int c = 0; c < n; ++c) cown[c0 + c] = b;
+    carry += ws[31];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) bchunk[NB] = carry;
+}
+
+// The same for more bins: counts, to be scanned into bchunk.
 static __global__ void k_bin_chunk_count(int NB, const int64_t *boff, int32_t *cnt) {
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < NB; b += gridDim.x * blockDim.x) {
     const long long n = boff[2 * b + 1] - boff[2 * b];

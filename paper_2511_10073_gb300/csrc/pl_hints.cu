@@ -571,19 +571,18 @@ __device__ __forceinline__ RowLen row_len(const LayIn &A, long long v) {
     else r.s = sl;
     return r;
   }
-  const long long sl = v < G.Nst ? A.srp[v + 1] - A.srp[v] : 0;
-  long long hl = 0, ws = 0;
-  bool virt = false;
-  if (v < G.C && A.hflag[v]) {
-    const int b = A.cell_bin[v];
-    hl = A.n_ovl[v];
+  // every load of the row is issued before any of them is looked at
+  const bool st = v < G.Nst, cell = v < G.C, mac = v >= G.mv0 && v < G.bn0;
+  const int64_t r0 = st ? A.srp[v] : 0, r1 = st ? A.srp[v + 1] : 0;
+  const uint8_t hf = cell ? A.hflag[v] : 0;
+  const int nov = cell ? A.n_ovl[v] : 0, b = cell ? A.cell_bin[v] : 0;
+  const int64_t m0 = mac ? A.moff[v - G.mv0] : 0, m1 = mac ? A.moff[v - G.mv0 + 1] : 0;
+  const long long sl = r1 - r0, hl = mac ? m1 - m0 : hf ? nov : 0;
+  const bool virt = v >= G.mv0;
+  // (the window slots in the grid matter, and are counted, only near the limit)
+  long long ws = 0;
+  if (hf && sl + hl <= kLong && sl + hl + (2 * G.hx + 1) * (2 * G.hy + 1) > kLong)
     ws = win_count(b % G.nbx, b / G.nbx, G);
-  } else if (v >= G.mv0 && v < G.bn0) {
-    hl = A.moff[v - G.mv0 + 1] - A.moff[v - G.mv0];
-    virt = true;
-  } else if (v >= G.bn0) {
-    virt = true;
-  }
   r.hub = virt || sl + hl + ws > kLong;
   if (r.hub) {
     r.l = (uint64_t)hl;
@@ -736,6 +735,9 @@ struct LayOut {
   const uint32_t *st_rp;
   const int32_t *st_longidx;
   const uint64_t *st_lptr;
+  int32_t *col;  // hint matrix: its entries, whose spare places are zeroed
+  void *w;
+  int wbytes;
 };
 // Rows alone (rp, srp, longidx): what is needed before the hub arrays' sizes
 // are known.  HUBS: the hub arrays too.
@@ -821,7 +823,14 @@ __global__ void __launch_bounds__(256) k_lay_apply(LayIn A, LayOut O, const LayS
     if (ROWS && !HINT && v <= A.G.Nst) O.srp[v] = (int64_t)(so + lo);
     o.s += __shfl_sync(0xffffffffu, x, 31);
   }
-  if (blockIdx.x != gridDim.x - 1 || threadIdx.x > kRpPad) return;
+  if (blockIdx.x != gridDim.x - 1) return;
+  if (HINT && threadIdx.x < kPad) {
+    const unsigned long long e = ns + tot->l + threadIdx.x;
+    O.col[e] = 0;
+    if (O.wbytes == 2) reinterpret_cast<uint16_t *>(O.w)[e] = 0;
+    else reinterpret_cast<uint32_t *>(O.w)[e] = 0u;
+  }
+  if (threadIdx.x > kRpPad) return;
   if (ROWS) {
     O.rp[N + threadIdx.x] = (uint32_t)ns;
   }
@@ -1355,37 +1364,35 @@ __global__ void k_lambda_max(int64_t N, const dfl *psum, unsigned long long *key
   if ((threadIdx.x & 31) == 0) atomicMax(key, best);
 }
 
-// lambda_up and 1 / lambda_up, also copied to status words 4..7 so that the
-// host reads them with the status.
-__global__ void k_lambda_final(double *lam, const unsigned long long *key, int *status) {
-  double l = df_from_maxkey(*key);
-  double il = 0.0;
-  if (!(l > 0.0) || isinf(l)) {
-    flag(status, ST_SPECTRUM);
-  } else {
-    il = __ddiv_rn(1.0, l);
+// lambda_up and 1 / lambda_up from the largest key (also copied to status words
+// 4..7, so that the host reads them with the status), then every row's
+// coefficient a_v = 1 - D_vv / lambda_up in FP32 and the hub rows' in FP64.
+__global__ void k_coef(int64_t N, const dfl *dsum, const unsigned long long *key, double *lam,
+                       int *status, float *c32, const uint32_t *pnlong, const int32_t *lrow,
+                       double *c64) {
+  __shared__ double s_il;
+  if (threadIdx.x == 0) {
+    const double l = df_from_maxkey(*key);
+    const bool ok = l > 0.0 && !isinf(l);
+    const double il = ok ? __ddiv_rn(1.0, l) : 0.0;
+    s_il = il;
+    if (blockIdx.x == 0) {
+      if (!ok) flag(status, ST_SPECTRUM);
+      lam[0] = l;
+      lam[1] = il;
+      reinterpret_cast<double *>(status + 4)[0] = l;
+      reinterpret_cast<double *>(status + 4)[1] = il;
+    }
   }
-  lam[0] = l;
-  lam[1] = il;
-  reinterpret_cast<double *>(status + 4)[0] = l;
-  reinterpret_cast<double *>(status + 4)[1] = il;
-}
-
-__global__ void k_coef(int64_t N, const dfl *dsum, const double *lam, float *c32) {
-  const float il = __double2float_rn(lam[1]);
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N;
-       v += (long long)gridDim.x * blockDim.x) {
+  __syncthreads();
+  const double ild = s_il;
+  const float il = __double2float_rn(ild);
+  const long long nlong = *pnlong, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x,
+                  nt = (long long)gridDim.x * blockDim.x;
+  for (long long l = t0; l < nlong; l += nt) c64[l] = 1.0 - df_to_d(dsum[lrow[l]]) * ild;
+  for (long long v = t0; v < N; v += nt) {
     dfl d = dsum[v];
     c32[v] = __fadd_rn(1.f, -__fmaf_rn(d.hi, il, __fmul_rn(d.lo, il)));
-  }
-}
-
-__global__ void k_coef_long(const uint32_t *pnlong, const int32_t *lrow, const dfl *dsum,
-                            const double *lam, double *c64) {
-  const int nlong = (int)*pnlong;
-  for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nlong; l += gridDim.x * blockDim.x) {
-    double d = df_to_d(dsum[lrow[l]]);
-    c64[l] = 1.0 - d * lam[1];
   }
 }
 
@@ -1530,12 +1537,14 @@ static LayOut lay_out(pl_graph *g, SpMat &m) {
   O.st_rp = P<uint32_t>(g->st.rp_s);
   O.st_longidx = P<int32_t>(g->st.longidx);
   O.st_lptr = P<uint64_t>(g->st.lptr);
+  O.col = P<int32_t>(m.col);
+  O.w = m.w.p;
+  O.wbytes = m.wbytes;
   return O;
 }
 
-// The entries' arrays (nnz of them and the spare ones, zeroed) and the arrays
-// over all rows.
-static pl_status lay_entries(pl_graph *g, SpMat &m, uint64_t nnz, cudaStream_t s) {
+// The entries' arrays (nnz of them and the spare ones) and the arrays over all rows.
+static pl_status lay_entries(pl_graph *g, SpMat &m, uint64_t nnz) {
   const int64_t N = g->N;
   const uint64_t cap = nnz + kPad;
   m.N = N;
@@ -1546,8 +1555,6 @@ static pl_status lay_entries(pl_graph *g, SpMat &m, uint64_t nnz, cudaStream_t s
   TRY(ensure(m.psum, (size_t)N * 8 + 16));
   TRY(ensure(m.c32, (size_t)N * 4 + 16));
   TRY(ensure(m.lam, 64));
-  TRY(cudaMemsetAsync(P<char>(m.col) + nnz * 4, 0, kPad * 4, s));
-  TRY(cudaMemsetAsync(P<char>(m.w) + nnz * m.wbytes, 0, kPad * m.wbytes, s));
   return PL_OK;
 }
 
@@ -1596,7 +1603,12 @@ pl_status prepare_static_layout(pl_graph *g, const int32_t *cnt, cudaStream_t s)
     TRY(cudaMemsetAsync(m.lchunk.p, 0, 4, s));
   }
   TRY(ensure(m.part, (size_t)(t.c + 1) * 16));
-  return lay_entries(g, m, t.s + t.l, s);
+  const uint64_t nnz = t.s + t.l;
+  st = lay_entries(g, m, nnz);
+  if (st != PL_OK) return st;
+  TRY(cudaMemsetAsync(P<char>(m.col) + nnz * 4, 0, kPad * 4, s));
+  TRY(cudaMemsetAsync(P<char>(m.w) + nnz * m.wbytes, 0, kPad * m.wbytes, s));
+  return PL_OK;
 }
 
 // Layout of the hint matrix for nml macro-cell overlaps, without a read by the
@@ -1615,7 +1627,7 @@ static pl_status layout_hints(pl_graph *g, const LayIn &A, int64_t nml, bool exa
   SpMat &m = g->hm;
   TRY(ensure(m.rp_s, (size_t)(N + 1 + kRpPad) * 4));
   TRY(ensure(m.longidx, (size_t)N * 4 + 16));
-  st = lay_entries(g, m, 2 * (uint64_t)nml, s);
+  st = lay_entries(g, m, 2 * (uint64_t)nml);
   if (st != PL_OK) return st;
   size_t nl = (size_t)g->Mm + g->NB + g->st.nlong + g->may_rows;
   size_t nc = nl + (size_t)((g->st.nnz_l + g->may_entries + 2 * (uint64_t)nml) / kChunk) + 1;
@@ -1840,8 +1852,26 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
       P<double>(g->amac), g->abin, p->capacity, p->mu, P<double>(g->Db), P<double>(g->Cb),
       P<double>(g->phi), phif, phil);
   note_launch();
+  // the bin rows' chunks, from the bucket starts
+  const long long nbc_max = nbl / kBinChunk + NB + 1;  // chunks at most (the grid size)
+  g->nbc_max = nbc_max;
+  TRY(ensure(g->bchunk, (size_t)(NB + 1) * 4 + 256));
+  TRY(ensure(g->cown, (size_t)nbc_max * 4 + 256));
+  if (NB <= kBinsOneBlock) {
+    k_bin_chunks<<<1, 1024, 0, s2>>>(NB, P<int64_t>(g->boff), P<int32_t>(g->bchunk), P<int32_t>(g->cown));
+    note_launch();
+  } else {
+    TRY(ensure(g->bcur, (size_t)(NB + 1) * 4 + 256));
+    TRY(ensure(g->tmp[5], scan_tmp_bytes(NB) + 4096));
+    int32_t *cnt = P<int32_t>(g->bcur);
+    k_bin_chunk_count<<<grid_for(NB, 256), 256, 0, s2>>>(NB, P<int64_t>(g->boff), cnt);
+    note_launch();
+    TRY((exclusive_scan<int32_t, int32_t>(cnt, P<int32_t>(g->bchunk), NB, g->tmp[5].p, s2)));
+    k_chunk_bins<<<grid_for(nbc_max, 256), 256, 0, s2>>>(NB, nbc_max, P<int32_t>(g->bchunk),
+                                                        P<int32_t>(g->cown));
+    note_launch();
+  }
   TRY(cudaEventRecord(g->ev_join, s2));
-  TRY(cudaEventRecord(g->ev_join2, s3));
   // H6-H7: row lengths and layout
   LayIn LA{};
   LA.G = G;
@@ -1854,7 +1884,6 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   size_t nl_max, nc_max;
   const int W = g->W;
   const size_t wb = g->wdtype == PL_W_BF16 ? 2 : 4;
-  const long long nbc_max = nbl / kBinChunk + NB + 1;  // bin-row chunks at most (the grid size)
   const size_t later = (size_t)C * (8 + W * wb + 4) + (size_t)(NB + 1) * 8 +
                        (size_t)nbc_max * (4 + kBinChunk * W * wb + 32 * W) + 16 * 512;
   pl_status st = layout_hints(g, LA, nml, cmem_ok || Mm == 0, later, s, &tot, &nl_max, &nc_max);
@@ -1865,8 +1894,9 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   TRY(ensure(g->mac_base, (size_t)C * 8 + 16));
   TRY(ensure(g->hbw, (size_t)C * W * m.wbytes + 64));
   TRY(ensure(g->hbin, (size_t)C * 4 + 16));
-  unsigned long long *counts = reinterpret_cast<unsigned long long *>(P<double>(m.lam) + 3);
-  TRY(cudaMemsetAsync(counts, 0, 16, s));
+  // the largest key (lambda_up), then the counts of window slots and hint cells
+  unsigned long long *key = reinterpret_cast<unsigned long long *>(P<double>(m.lam) + 2), *counts = key + 1;
+  TRY(cudaMemsetAsync(key, 0, 24, s));
   TRY(cudaStreamWaitEvent(s, g->ev_join, 0));  // phi
   (g->wdtype == PL_W_BF16 ? k_assemble_hints<true> : k_assemble_hints<false>)
       <<<grid_for(g->Nst, 256), 256, 0, s>>>(
@@ -1878,18 +1908,22 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
       g->hbw.p, P<int32_t>(g->hbin), P<dfl>(m.dsum), P<dfl>(m.psum), P<uint64_t>(g->mac_base),
       counts);
   note_launch();
-  // H10: bin rows (degree partials of the window blocks, chunk by chunk) and
-  // macro rows (their entries and degree partials)
+  // macro rows (their entries and degree partials) on the third stream, behind
+  // the macro lists there, beside the bin rows' blocks and degrees here
+  TRY(ensure(g->tmp[5], (nc_max + 1) * 2 * sizeof(dfl) + 256));
+  dfl *cpart = P<dfl>(g->tmp[5]);
+  TRY(cudaEventRecord(g->ev_fork, s));
+  TRY(cudaStreamWaitEvent(s3, g->ev_fork, 0));
+  if (nc_max) {
+    k_hub_chunks<<<(int)(nc_max < 152 * 32 ? nc_max : 152 * 32), 256, 0, s3>>>(
+        G, g->wdtype, &tot->c, P<int32_t>(m.chunk_lr), P<int32_t>(m.lrow), P<uint64_t>(m.lptr),
+        P<int32_t>(m.lchunk), P<int64_t>(g->moff), P<uint32_t>(g->mlist), P<int32_t>(g->n_ovl),
+        P<uint64_t>(g->mac_base), P<int32_t>(m.col), m.w.p, cpart);
+    note_launch();
+  }
+  TRY(cudaEventRecord(g->ev_join2, s3));
+  // H10: bin rows (degree partials of the window blocks, chunk by chunk)
   const BinGeo B = make_bingeo(g);
-  TRY(ensure(g->bchunk, (size_t)(NB + 1) * 4 + 256));
-  TRY(ensure(g->tmp[6], (size_t)(NB + 1) * 4 + 256));
-  k_bin_chunk_count<<<grid_for(NB, 256), 256, 0, s>>>(NB, P<int64_t>(g->boff), P<int32_t>(g->tmp[6]));
-  note_launch();
-  TRY((exclusive_scan<int32_t, int32_t>(P<int32_t>(g->tmp[6]), P<int32_t>(g->bchunk), NB, stmp, s)));
-  g->nbc_max = nbc_max;
-  TRY(ensure(g->cown, (size_t)nbc_max * 4 + 256));
-  k_chunk_bins<<<grid_for(nbc_max, 256), 256, 0, s>>>(NB, nbc_max, P<int32_t>(g->bchunk), P<int32_t>(g->cown));
-  note_launch();
   // the chunks' copy of the window blocks (read slot by slot by the bin rows)
   TRY(ensure(g->hbwq, (size_t)nbc_max * kBinChunk * W * m.wbytes + 64));
   {
@@ -1912,16 +1946,7 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
                                  P<int64_t>(g->boff), P<uint32_t>(g->blist), g->hbwq.p, nullptr,
                                  P<float4>(g->bdeg)));
   note_launch();
-  TRY(ensure(g->tmp[5], (nc_max + 1) * 2 * sizeof(dfl) + 256));
-  dfl *cpart = P<dfl>(g->tmp[5]);
-  TRY(cudaStreamWaitEvent(s, g->ev_join2, 0));  // the macro lists
-  if (nc_max) {
-    k_hub_chunks<<<(int)(nc_max < 152 * 32 ? nc_max : 152 * 32), 256, 0, s>>>(
-        G, g->wdtype, &tot->c, P<int32_t>(m.chunk_lr), P<int32_t>(m.lrow), P<uint64_t>(m.lptr),
-        P<int32_t>(m.lchunk), P<int64_t>(g->moff), P<uint32_t>(g->mlist), P<int32_t>(g->n_ovl),
-        P<uint64_t>(g->mac_base), P<int32_t>(m.col), m.w.p, cpart);
-    note_launch();
-  }
+  TRY(cudaStreamWaitEvent(s, g->ev_join2, 0));
   if (nl_max) {
     k_hub_finalize<<<grid_for((long long)nl_max * 32, 256), 256, 0, s>>>(
         G, B, &tot->f, P<int32_t>(m.lrow), P<int32_t>(m.lchunk), cpart, P<int32_t>(g->bchunk),
@@ -1930,19 +1955,13 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
     note_launch();
   }
   // H11: lambda_up and coefficients
-  unsigned long long *key = reinterpret_cast<unsigned long long *>(P<double>(m.lam) + 2);
-  TRY(cudaMemsetAsync(key, 0, 8, s));
   k_lambda_max<<<grid_for(N, 256, 152 * 8), 256, 0, s>>>(N, P<dfl>(m.psum), key);
   note_launch();
-  k_lambda_final<<<1, 1, 0, s>>>(P<double>(m.lam), key, status);
+  // (one wave of blocks: each forms 1 / lambda_up once)
+  k_coef<<<grid_for(N, 256, 152 * 8), 256, 0, s>>>(N, P<dfl>(m.dsum), key, P<double>(m.lam), status,
+                                                  P<float>(m.c32), &tot->f, P<int32_t>(m.lrow),
+                                                  P<double>(m.c64l));
   note_launch();
-  k_coef<<<grid_for(N, 256), 256, 0, s>>>(N, P<dfl>(m.dsum), P<double>(m.lam), P<float>(m.c32));
-  note_launch();
-  if (nl_max) {
-    k_coef_long<<<grid_for((long long)nl_max, 256), 256, 0, s>>>(&tot->f, P<int32_t>(m.lrow), P<dfl>(m.dsum),
-                                                        P<double>(m.lam), P<double>(m.c64l));
-    note_launch();
-  }
   TRY(cudaGetLastError());
   {
     unsigned long long ns[2] = {0, 0};

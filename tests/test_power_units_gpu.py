@@ -25,6 +25,8 @@ CASES = {
     "no_macros": (500, [2] * 400 + [5] * 60, dict(nbx=16, nby=16)),
     "one_cell": (2, [2], dict(nbx=5, nby=3)),
     "long_rows": (600, [16] * 350 + [40] * 3 + [300], dict(nbx=32, nby=32)),
+    # more bins than one block numbers the chunks of
+    "bins_18000": (300, [3] * 250, dict(nbx=150, nby=120)),
     "many_bins": (900, [3] * 800, dict(nbx=64, nby=64)),
 }
 
