@@ -975,9 +975,15 @@ __device__ __forceinline__ float df_weight(dfl e, dfl w, float tol, bool *tie) {
 // weight itself is a double-float (exponential to 2^-42, products to 2^-45): its
 // FP64 form, at 1/64 of the FP32 rate, took 352 us of a 210k-cell design's refinement
 // round of 970 us (order 8); with the double-float form the round takes 641 us.
-constexpr int kAsmStage = 752;  // own entries of a warp's 32 rows staged in shared memory
+// Own entries and window blocks of a warp's 32 rows are staged in shared memory
+// and written as one run each: a block is W weights at a stride of W per lane,
+// which as plain stores are W partial writes of several lines.  2.2M cells, BF16,
+// 3 x 3 windows: 173 -> 169 us, and 146 us with the four blocks per SM that the
+// smaller stage leaves room for (FP32 storage: 25 us with three, 28 with four).
+constexpr int kAsmStage = 256;   // entries
+constexpr int kAsmBlock = 2304;  // bytes of window blocks (wider windows are written directly)
 template <bool bf>
-__global__ void __launch_bounds__(256, 3) k_assemble_hints(
+__global__ void __launch_bounds__(256, bf ? 4 : 3) k_assemble_hints(
     HintGeo G, ExpTable xt, const uint32_t *hrp, const int32_t *longidx, const uint64_t *lptr,
     const dfl *sdsum, const dfl *spsum, const uint8_t *hflag, const int32_t *cell_bin,
     const int32_t *n_ovl, const float2 *xy, const float *cw, const float *ch,
@@ -995,6 +1001,10 @@ __global__ void __launch_bounds__(256, 3) k_assemble_hints(
   const int lane = threadIdx.x & 31;
   int32_t *scol = stage_col[threadIdx.x >> 5];
   uint32_t *sw = stage_w[threadIdx.x >> 5];
+  __shared__ __align__(16) uint8_t stage_blk[8][kAsmBlock];
+  uint8_t *sblk = stage_blk[threadIdx.x >> 5];
+  constexpr int wbytes = bf ? 2 : 4;
+  const bool sb = 32 * W * wbytes <= kAsmBlock;
   const long long stride = (long long)gridDim.x * blockDim.x;
   unsigned long long slots = 0, hints = 0;  // this thread's window slots in the grid, hint cells
   for (long long v0 = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); v0 < G.Nst;
@@ -1098,8 +1108,10 @@ __global__ void __launch_bounds__(256, 3) k_assemble_hints(
       const int b = cb, bx = b % G.nbx, by = b / G.nbx, wx = 2 * G.hx + 1;
       const dfl ux = df_offset_scale(p.x, G.xlh, G.xll, G.iwh, G.iwl);
       const dfl uy = df_offset_scale(p.y, G.ylh, G.yll, G.ihh, G.ihl);
-      uint16_t *wb16 = reinterpret_cast<uint16_t *>(bwin) + (size_t)v * W;
-      uint32_t *wb32 = reinterpret_cast<uint32_t *>(bwin) + (size_t)v * W;
+      uint16_t *wb16 = sb ? reinterpret_cast<uint16_t *>(sblk) + lane * W
+                          : reinterpret_cast<uint16_t *>(bwin) + (size_t)v * W;
+      uint32_t *wb32 = sb ? reinterpret_cast<uint32_t *>(sblk) + lane * W
+                          : reinterpret_cast<uint32_t *>(bwin) + (size_t)v * W;
       int sidx = 0;
       if (bf && G.hx == 1) {
         // three window columns: their ratios and e^{-rx} once per cell, not
@@ -1221,7 +1233,18 @@ __global__ void __launch_bounds__(256, 3) k_assemble_hints(
     psum[v] = df_norm(Pl);
     }
   flush:
-    // the staged range, written with coalesced stores
+    // the staged blocks and entries, written with coalesced stores (the block of a
+    // cell without hints is never read; whatever the stage held goes there)
+    if (sb && v0 < G.C) {
+      __syncwarp();
+      const int nb = (int)(min((long long)32, G.C - v0) * W * wbytes);
+      uint8_t *dst = reinterpret_cast<uint8_t *>(bwin) + (size_t)v0 * W * wbytes;
+      for (int i = lane * 4; i + 4 <= nb; i += 128)
+        *reinterpret_cast<uint32_t *>(dst + i) = *reinterpret_cast<const uint32_t *>(sblk + i);
+      if ((nb & 2) && lane == 0)
+        *reinterpret_cast<uint16_t *>(dst + nb - 2) = *reinterpret_cast<const uint16_t *>(sblk + nb - 2);
+      __syncwarp();
+    }
     if (staged) {
       __syncwarp();
       for (uint64_t i = lane; i < re - rb; i += 32) {
