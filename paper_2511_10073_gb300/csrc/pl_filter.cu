@@ -682,9 +682,6 @@ __global__ void __launch_bounds__(kHubRows * 32) k_hub_rows(StepArgs A) {
 // completion before they touch memory.  A launch lets its own dependents in only
 // after that wait, so no more than one launch is ever ahead, and x is read with
 // coherent loads (it is written while a waiting launch already exists).
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;"); }
-
 template <int WT, bool NINE>
 __global__ void __launch_bounds__(256, 4) k_power_units(StepArgs A, long long nbin) {
   pdl_wait();
@@ -896,21 +893,6 @@ static int graph_nsm(pl_graph *g) {
   return g->nsm;
 }
 
-// Launches kernel k as a programmatic dependent of the launch before it on s.
-template <typename... P, typename... Q>
-static cudaError_t launch_pdl(void (*k)(P...), int grid, int block, cudaStream_t s, Q... args) {
-  cudaLaunchConfig_t c{};
-  c.gridDim = dim3((unsigned)grid);
-  c.blockDim = dim3((unsigned)block);
-  c.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  c.attrs = &at;
-  c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, k, P(args)...);
-}
-
 // Blocks of k_power_units per SM up to which a refinement product takes that
 // form.  Above, the short rows' own kernel (40 registers, one persistent wave)
 // beside the hub and bin kernels on the second stream is the better one.  A round
@@ -932,10 +914,10 @@ static cudaError_t launch_step(const StepArgs &A, double bytes, int wdtype, cuda
       const bool bf = wdtype == PL_W_BF16, nine = A.B.W == 9;
       auto ku = bf ? (nine ? k_power_units<1, true> : k_power_units<1, false>)
                    : (nine ? k_power_units<0, true> : k_power_units<0, false>);
-      cudaError_t e = launch_pdl(ku, (int)blocks, 256, s, A, nbin);
+      cudaError_t e = launch_pdl(ku, (int)blocks, 256, 0, s, A, nbin);
       if (e == cudaSuccess)
         e = launch_pdl(bf ? k_power_hubs<1> : k_power_hubs<0>, (A.nlong + kHubRows - 1) / kHubRows,
-                       kHubRows * 32, s, A);
+                       kHubRows * 32, 0, s, A);
       note_launch();
       note_launch();
       if (prof) prof_end(s);

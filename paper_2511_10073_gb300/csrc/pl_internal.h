@@ -251,3 +251,30 @@ inline cudaError_t ensure_side2(pl_graph *g) {
   return e;
 }
 }  // namespace pl
+
+namespace pl {
+#ifdef __CUDACC__
+// Programmatic dependent launches: a kernel launched by launch_pdl may be
+// placed while the launch before it on its stream still runs; pdl_wait waits
+// for that one's completion and its writes.  Every thread calls it before it
+// touches memory that the launch before may write or read, and pdl_release
+// only after it, so that no more than one launch is ever ahead.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;"); }
+template <typename... P, typename... Q>
+inline cudaError_t launch_pdl(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s,
+                              Q... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)block);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+#endif
+}  // namespace pl

@@ -185,23 +185,23 @@ __device__ __forceinline__ uint8_t *smem_base() {
 __device__ uint32_t tc_setup(uint8_t *sm, const float *w) {
   const int t = threadIdx.x;
   for (int i = t; i < kHid * kNF; i += kTile)
-    *reinterpret_cast<uint16_t *>(sm + SM_W1 + opnd_off(i / kNF, i % kNF, 0)) = f2bf16(w[kW1 + i]);
+    *reinterpret_cast<uint16_t *>(sm + SM_W1 + opnd_off(i / kNF, i % kNF, 0)) = f2bf16(__ldcg(w + kW1 + i));
   float *w2f = reinterpret_cast<float *>(sm + SM_W2F);
   for (int i = t; i < kN2 * kHid; i += kTile) {
     const int n = i / kHid, j = i % kHid;
-    const uint16_t b = n < kNOut ? f2bf16(w[kW2 + n * kHid + j]) : (uint16_t)0;
+    const uint16_t b = n < kNOut ? f2bf16(__ldcg(w + kW2 + n * kHid + j)) : (uint16_t)0;
     *reinterpret_cast<uint16_t *>(sm + SM_W2 + opnd_off(n, j, 512)) = b;
     if (n < kNOut) w2f[j * kNOut + n] = bf16_to_f(b);
   }
   float *b1 = reinterpret_cast<float *>(sm + SM_B1);
   float *prm = reinterpret_cast<float *>(sm + SM_PRM);
-  if (t < kHid) b1[t] = w[kB1 + t];
+  if (t < kHid) b1[t] = __ldcg(w + kB1 + t);
   if (t < kNF) {
-    prm[t] = w[kMU + t];
-    prm[16 + t] = w[kISD + t];
+    prm[t] = __ldcg(w + kMU + t);
+    prm[16 + t] = __ldcg(w + kISD + t);
   }
-  if (t < 3) prm[32 + t] = w[kTH + t];
-  if (t < kNOut) prm[36 + t] = w[kB2 + t];
+  if (t < 3) prm[32 + t] = __ldcg(w + kTH + t);
+  if (t < kNOut) prm[36 + t] = __ldcg(w + kB2 + t);
   const uint32_t bar = su32(sm + SM_BAR);
   if (t == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
@@ -602,7 +602,10 @@ __global__ void __launch_bounds__(kTile) k_train_tile(const float *rec, int64_t 
     for (int k = 0; k < kNF; ++k) q.f[k] = 0.f;
     q.G[0][0] = q.G[0][1] = q.G[1][0] = q.G[1][1] = q.G[2][0] = q.G[2][1] = q.T[0] = q.T[1] = 0.f;
   }
-  // the record's loads are in flight during the setup
+  // the record's loads are in flight during the wait for the step before (whose
+  // weights this one reads, and whose gradient rows it overwrites) and the setup
+  pdl_wait();
+  pdl_release();
   const uint32_t tmem = tc_setup(sm, w);
   const float *prm = reinterpret_cast<const float *>(sm + SM_PRM);
   uint32_t xw[8];
@@ -743,7 +746,7 @@ __device__ __forceinline__ double sum_parts(const float *part, int nblk, double 
   for (int b = seg * per; b < b1; b += 16) {
     float v[16];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) v[u] = b + u < b1 && i < kPart ? part[(int64_t)(b + u) * kPart + i] : 0.f;
+    for (int u = 0; u < 16; ++u) v[u] = b + u < b1 && i < kPart ? __ldcg(part + (int64_t)(b + u) * kPart + i) : 0.f;
 #pragma unroll
     for (int u = 0; u < 16; ++u) s += f2d(v[u]);
   }
@@ -772,6 +775,8 @@ __global__ void __launch_bounds__(32 * kSegs) k_adam(const float *part, int nblk
                                                      float *v, float lr, float b1, float b2,
                                                      float eps, float bc1, float bc2, double *loss) {
   __shared__ double sh[kSegs][32];
+  pdl_wait();
+  pdl_release();
   const double s = sum_parts(part, nblk, sh);
   const int i = kTH + blockIdx.x * 32 + threadIdx.x;
   if (threadIdx.x >= 32 || i > kLW) return;
@@ -785,7 +790,7 @@ __global__ void __launch_bounds__(32 * kSegs) k_adam(const float *part, int nblk
   const float vi = __fmaf_rn(b2, v[i], __fmul_rn(__fmul_rn(1.f - b2, g), g));
   m[i] = mi;
   v[i] = vi;
-  w[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+  w[i] = __ldcg(w + i) - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
 }
 
 __global__ void k_acc_to_grad(const double *acc, float *grad) {
@@ -1271,12 +1276,18 @@ pl_status pl_learned_train(const float *rec, int64_t nrec, float *w, const pl_tr
       const double lr = o->lr_min + 0.5 * (o->lr - o->lr_min) *
                                         (1.0 + std::cos(3.14159265358979323846 * (double)step / (double)total));
       const double t = (double)(step + 1);
-      k_train_tile<<<bt, kTile, kSmemTrain, s>>>(rec, nrec, W.tiles + k * bt, 0,
-                                                1.f / (float)(bt * kTile), w, W.part, status);
-      k_adam<<<kPartGrid, 32 * kSegs, 0, s>>>(W.part, bt, w, W.m, W.v, (float)lr, (float)o->beta1,
-                                              (float)o->beta2, (float)o->eps,
-                                              (float)(1.0 - std::pow(o->beta1, t)),
-                                              (float)(1.0 - std::pow(o->beta2, t)), W.loss);
+      // an epoch's first launch follows copies and clears in full, the others are
+      // programmatic dependents of the one before (two epochs over 630k records:
+      // 1859 -> 1657 us)
+      if (k == 0)
+        k_train_tile<<<bt, kTile, kSmemTrain, s>>>(rec, nrec, W.tiles, 0, 1.f / (float)(bt * kTile), w,
+                                                  W.part, status);
+      else
+        TRY(launch_pdl(k_train_tile, bt, kTile, kSmemTrain, s, rec, nrec, W.tiles + k * bt, (int64_t)0,
+                       1.f / (float)(bt * kTile), w, W.part, status));
+      TRY(launch_pdl(k_adam, kPartGrid, 32 * kSegs, 0, s, W.part, bt, w, W.m, W.v, (float)lr,
+                     (float)o->beta1, (float)o->beta2, (float)o->eps,
+                     (float)(1.0 - std::pow(o->beta1, t)), (float)(1.0 - std::pow(o->beta2, t)), W.loss));
       note_launch();
       note_launch();
     }
