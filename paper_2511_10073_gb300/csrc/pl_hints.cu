@@ -1706,7 +1706,7 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
     // (the counts of a workspace with little room left: the largest tiles)
     const Arena *ar = current_arena();
     const uint64_t nt = std::max<uint64_t>(1, ((uint64_t)C + (1u << tsh) - 1) >> tsh);
-    if ((nt * ((uint64_t)Mm + 2 * (uint64_t)NB)) * 12 > (ar->cap - ar->used) / 4) tsh = 12;
+    if ((nt * ((uint64_t)Mm + 2 * (uint64_t)NB)) * 12 > (ar->cap - ar->used) / 16) tsh = 12;
   }
   const int ntile = std::max(1, (int)(((int64_t)C + (1 << tsh) - 1) >> tsh));
   // macro lists by a tiled counting sort when the macros' run counters fit
