@@ -232,8 +232,8 @@ __device__ __forceinline__ void epilogue(const StepArgs &A, int64_t v, T yx, T y
 
 // ------------------------------------------------------- work units
 // Hub chunks [0, nchunks) of kChunk entries (first launch), hub rows (second
-// launch), then the short rows (third launch); warps take units gw,
-// gw + nwarps, ... and no unit needs a block-wide barrier.
+// launch), then the short rows (third launch); hub chunks are dealt to the warps
+// in turn, and no unit needs a block-wide barrier.
 //  * hub chunk: exact products accumulated in double-float, reduced over the
 //    warp, written as a double-float partial;
 //  * hub row: the row's partials added by a warp in a fixed order, then
@@ -527,7 +527,9 @@ template <int WT, int MODE>
 __global__ void __launch_bounds__(kRowThreads, 6) k_spmm_rows(StepArgs A) {
   constexpr int RPW = 32 / kRowLanes, WPB = kRowThreads / 32;
   const int wid = threadIdx.x >> 5;
-  // cells: a run of consecutive row groups per block
+  // cells: a run of consecutive row groups per block, so that the neighbours'
+  // coordinates (mostly within a few thousand cells) stay in the SM's L1 (a round
+  // of 2.2M cells: 2239 us with the groups dealt to the blocks in turn, 2195 us)
   const long long nc = A.C / RPW, per = (nc + gridDim.x - 1) / gridDim.x;
   const long long c0 = blockIdx.x * per, c1 = c0 + per < nc ? c0 + per : nc;
   for (long long k = c0 + wid; k < c1; k += WPB) rows_group<WT, MODE>(A, k * RPW);
