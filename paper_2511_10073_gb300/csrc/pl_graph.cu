@@ -1031,6 +1031,7 @@ pl_status build_static(pl_graph *g, const pl_netlist *nl, const pl_params *p, cu
     g->star_w_ok = true;
   }
   TRY(ensure_side(g));
+  SideJoin join{g, s, true};
   TRY(cudaEventRecord(g->ev_fork, s));
   TRY(cudaStreamWaitEvent(g->side, g->ev_fork, 0));
   {
@@ -1166,6 +1167,7 @@ pl_status build_static(pl_graph *g, const pl_netlist *nl, const pl_params *p, cu
   g->gsy = sy;
   TRY(cudaEventRecord(g->ev_join, s2));
   TRY(cudaStreamWaitEvent(s, g->ev_join, 0));
+  join.armed = false;
   TRY(cudaGetLastError());
   TRY(cudaStreamSynchronize(s));
   g->nnz_static = g->st.nnz_s + g->st.nnz_l;

@@ -1826,6 +1826,7 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   TRY(ensure(g->phi, (size_t)NB * 8 + 16));
   TRY(ensure(g->tmp[4], (size_t)NB * 8 + 256));
   float *phif = P<float>(g->tmp[4]), *phil = phif + NB;  // phi_b as double-floats
+  SideJoin join{g, s, true};
   TRY(cudaEventRecord(g->ev_fork, s));
   TRY(cudaStreamWaitEvent(s2, g->ev_fork, 0));
   TRY(cudaStreamWaitEvent(s3, g->ev_fork, 0));
@@ -1970,6 +1971,7 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
                                  P<float4>(g->bdeg)));
   note_launch();
   TRY(cudaStreamWaitEvent(s, g->ev_join2, 0));
+  join.armed = false;
   if (nl_max) {
     k_hub_finalize<<<grid_for((long long)nl_max * 32, 256), 256, 0, s>>>(
         G, B, &tot->f, P<int32_t>(m.lrow), P<int32_t>(m.lchunk), cpart, P<int32_t>(g->bchunk),

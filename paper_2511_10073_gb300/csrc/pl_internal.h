@@ -250,6 +250,21 @@ inline cudaError_t ensure_side2(pl_graph *g) {
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->ev_join2, cudaEventDisableTiming);
   return e;
 }
+// A call that has forked work onto the graph's side streams and leaves before its
+// own joins (a workspace that runs out between them) joins them here: the given
+// stream covers every kernel of the call on each way out of it.
+struct SideJoin {
+  pl_graph *g;
+  cudaStream_t s;
+  bool armed;
+  ~SideJoin() {
+    if (!armed) return;
+    if (g->side && cudaEventRecord(g->ev_join, g->side) == cudaSuccess)
+      cudaStreamWaitEvent(s, g->ev_join, 0);
+    if (g->side2 && cudaEventRecord(g->ev_join2, g->side2) == cudaSuccess)
+      cudaStreamWaitEvent(s, g->ev_join2, 0);
+  }
+};
 }  // namespace pl
 
 namespace pl {
