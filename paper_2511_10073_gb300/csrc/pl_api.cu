@@ -204,10 +204,12 @@ pl_status pl_build_graph(const pl_netlist *nl, const pl_params *p, const float *
     *gp = new (std::nothrow) pl_graph();
     if (!*gp) { set_error("host allocation failed"); return PL_ERR_OOM; }
     created = true;
-  } else if ((*gp)->stream) {
-    // the previous build's work on its streams ends before its memory is reused
+  } else {
+    // what earlier calls left on any of the graph's streams (the given one may be
+    // the legacy default stream, NULL) ends before its memory is reused
     cudaStreamSynchronize((*gp)->stream);
     if ((*gp)->side) cudaStreamSynchronize((*gp)->side);
+    if ((*gp)->side2) cudaStreamSynchronize((*gp)->side2);
   }
   pl_graph *g = *gp;
   for_each_buf(g, 0, [](Buf &b) { release(b); });

@@ -67,3 +67,28 @@ def test_a_failed_build_is_covered_by_its_stream(own_stream):
         pl.pl_build_hints(g, prm, xy)
         pl.pl_filter_apply(g, prm, xy, out)
         assert torch.equal(out, want)
+
+
+def test_a_rebuild_waits_for_what_was_queued_on_the_default_stream():
+    """A call that does not synchronize, queued on the default stream (NULL) behind
+    other work, reads the graph's workspace after a rebuild of the graph on
+    another stream was asked for."""
+    import paper_2511_10073_gb300 as pl
+    dnl = pl.DeviceNetlist(netgen.make_netlist("medium", 1))
+    other = pl.DeviceNetlist(netgen.make_netlist("medium", 2))
+    prm = pl.params(nbx=32, nby=32)
+    ws = pl.workspace(max(pl.pl_workspace_size(d, prm) for d in (dnl, other)))
+    with torch.cuda.stream(torch.cuda.default_stream()):
+        g = pl.pl_build_graph(dnl, prm, ws=ws)
+        want = torch.empty(g.info()["N"] * 2, dtype=torch.float32, device="cuda")
+        out = torch.zeros_like(want)
+        pl.pl_init_signal(g, 1, None, want)
+        a = torch.ones((8192, 8192), device="cuda")
+        torch.cuda.synchronize()
+        for _ in range(4):
+            a @ a
+        pl.pl_init_signal(g, 1, None, out)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        pl.pl_build_graph(other, prm, graph=g, ws=ws)
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
