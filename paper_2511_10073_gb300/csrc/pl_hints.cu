@@ -1672,7 +1672,10 @@ static pl_status layout_hints(pl_graph *g, const LayIn &A, int64_t nml, bool exa
   return PL_OK;
 }
 
-pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaStream_t s) {
+// tight: the largest tiles of the counting sorts and exact hub counts, which
+// take the least memory.
+static pl_status build_hints_in(pl_graph *g, const pl_params *p, const float *xy_in, bool tight,
+                                cudaStream_t s) {
   const int64_t N = g->N;
   const int32_t C = g->C, NB = g->NB, Mm = g->Mm;
   const float2 *xy = reinterpret_cast<const float2 *>(xy_in);
@@ -1701,9 +1704,10 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   TRY(ensure(g->bcnt, (size_t)(nbk + 1) * 4));
   TRY(ensure(g->mcnt, (size_t)(Mm + 1) * 4));
   if (!tiled) TRY(cudaMemsetAsync(g->bcnt.p, 0, (size_t)(nbk + 1) * 4, s));
-  int tsh = hint_tile_shift(C, NB, Mm);
+  int tsh = tight ? 12 : hint_tile_shift(C, NB, Mm);
   {
-    // (the counts of a workspace with little room left: the largest tiles)
+    // (in a workspace whose rest the counts would take a good part of: the largest
+    // tiles, so that the build need not be repeated with them)
     const Arena *ar = current_arena();
     const uint64_t nt = std::max<uint64_t>(1, ((uint64_t)C + (1u << tsh) - 1) >> tsh);
     if ((nt * ((uint64_t)Mm + 2 * (uint64_t)NB)) * 12 > (ar->cap - ar->used) / 16) tsh = 12;
@@ -1910,7 +1914,7 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
   const size_t wb = g->wdtype == PL_W_BF16 ? 2 : 4;
   const size_t later = (size_t)C * (8 + W * wb + 4) + (size_t)(NB + 1) * 8 +
                        (size_t)nbc_max * (4 + kBinChunk * W * wb + 32 * W) + 16 * 512;
-  pl_status st = layout_hints(g, LA, nml, cmem_ok || Mm == 0, later, s, &tot, &nl_max, &nc_max);
+  pl_status st = layout_hints(g, LA, nml, !tight && (cmem_ok || Mm == 0), later, s, &tot, &nl_max, &nc_max);
   if (st != PL_OK) return st;
   SpMat &m = g->hm;
   // H9: hint parts of cells (macro entries, window blocks) and degrees of
@@ -2005,6 +2009,15 @@ pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy_in, cudaS
     return PL_ERR_SPECTRUM;
   }
   return PL_OK;
+}
+
+// A workspace that does not hold the build with its quicker, larger tables is
+// refused only when it does not hold the smallest one either.
+pl_status build_hints(pl_graph *g, const pl_params *p, const float *xy, cudaStream_t s) {
+  const pl_status st = build_hints_in(g, p, xy, false, s);
+  if (st != PL_ERR_WORKSPACE) return st;
+  g->arena.short_need = 0;
+  return build_hints_in(g, p, xy, true, s);
 }
 
 }  // namespace pl

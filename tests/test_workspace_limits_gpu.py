@@ -92,3 +92,42 @@ def test_a_rebuild_waits_for_what_was_queued_on_the_default_stream():
         pl.pl_build_graph(other, prm, graph=g, ws=ws)
     torch.cuda.synchronize()
     assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("wd", [1, 2])
+def test_small_tiles_do_not_cost_a_workspace(wd):
+    """A design whose counting sorts take tiles of 1024 cells where there is room:
+    workspaces that hold the build only with tiles of 4096 cells (12 bytes for
+    each tile and bucket or macro) suffice too, and a size that suffices is not
+    followed by a larger one that does not."""
+    import paper_2511_10073_gb300 as pl
+    nl = netgen.make_netlist("medium", 1)
+    dnl = pl.DeviceNetlist(nl)
+    prm = pl.params(nbx=10, nby=10, det_ratio=0.5, wdtype=wd)
+    g = pl.pl_build_graph(dnl, prm)
+    xy = torch.empty(g.info()["N"] * 2, dtype=torch.float32, device="cuda")
+    pl.pl_init_signal(g, 1, None, xy)
+    pl.pl_build_hints(g, prm, xy)
+    want, out = torch.empty_like(xy), torch.empty_like(xy)
+    pl.pl_filter_apply(g, prm, xy, want)
+    info = g.info()
+    counts = lambda tile: -(-nl.num_cells // tile) * (info["macros"] + 2 * info["bins"]) * 12
+    extra = counts(1024) - counts(4096)
+    assert counts(1024) * 16 + 4 * extra < info["ws_peak"] - info["ws_static"]  # small tiles are taken
+    fits = []
+    for less in [4 * extra, 2 * extra, extra - (1 << 16), extra // 2, 1 << 16, 4096, 0]:
+        h = _build(pl, dnl, prm, ws=pl.workspace(info["ws_peak"] - less))
+        if h is None:
+            fits.append(False)
+            continue
+        try:
+            pl.pl_build_hints(h, prm, xy)
+        except pl.PlError as e:
+            assert e.code == pl.PL_ERR_WORKSPACE
+            fits.append(False)
+            continue
+        pl.pl_filter_apply(h, prm, xy, out)
+        assert torch.equal(out, want)
+        fits.append(True)
+    assert all(fits[2:])
+    assert fits == sorted(fits)
