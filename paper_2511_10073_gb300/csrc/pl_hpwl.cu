@@ -24,36 +24,37 @@ constexpr int kHpwlGrid = 152 * kHpwlPerSm;     // what is launched: one wave of
 constexpr int kHpwlWin = 256;        // pins a warp stages at once
 constexpr int kHpwlLane = 16;        // pins of a window that one lane spans
 constexpr int kHpwlWarpMax = 1024;   // longer nets are spanned by a whole block
-constexpr int kHpwlBigs = 8;         // such nets a warp keeps for its block
+constexpr int kHpwlList = 31;        // such nets a warp keeps a list of
 
-// Positions of pins k0, k0 + stride, ... (kPins of them, those below e): all
+// Positions of pins k0, k0 + stride, ... (n of them, those below e): all
 // cell indices and offsets are loaded, then all cells gathered.  A pin_cell
 // outside [0, C) sets bad and reads cell 0 instead (the call then reports NaN):
 // nothing is written or branched on between the loads, so they stay in flight
 // together.
-constexpr int kPins = 4;
+constexpr int kPins = 4;  // of a window
+template <int n>
 __device__ __forceinline__ void pin_pos(const float2 *xy, const int32_t *pin_cell, const float *dx,
                                         const float *dy, long long k0, int stride, long long e,
                                         int32_t C, bool &bad, float2 *p) {
-  int32_t c[kPins];
-  float ox[kPins], oy[kPins];
+  int32_t c[n];
+  float ox[n], oy[n];
 #pragma unroll
-  for (int u = 0; u < kPins; ++u) {
+  for (int u = 0; u < n; ++u) {
     const long long k = k0 + (long long)u * stride;
     const bool in = k < e;
-    c[u] = in ? __ldcs(pin_cell + k) : 0;
-    ox[u] = in && dx ? __ldcs(dx + k) : 0.f;
-    oy[u] = in && dy ? __ldcs(dy + k) : 0.f;
+    c[u] = in ? __ldg(pin_cell + k) : 0;
+    ox[u] = in && dx ? __ldg(dx + k) : 0.f;
+    oy[u] = in && dy ? __ldg(dy + k) : 0.f;
   }
 #pragma unroll
-  for (int u = 0; u < kPins; ++u) {
+  for (int u = 0; u < n; ++u) {
     const bool ok = (uint32_t)c[u] < (uint32_t)C;
     const bool in = k0 + (long long)u * stride < e;
     bad |= in && !ok;
     p[u] = in && C > 0 ? xy[ok ? c[u] : 0] : make_float2(0.f, 0.f);
   }
 #pragma unroll
-  for (int u = 0; u < kPins; ++u) {
+  for (int u = 0; u < n; ++u) {
     if (dx) p[u].x += ox[u];
     if (dy) p[u].y += oy[u];
   }
@@ -96,17 +97,17 @@ struct Extent {
   }
 };
 
-// This thread's share of pins [b, e) (every nt-th from t), kPins gathers in flight.
+// This thread's share of pins [b, e) (every nt-th from t), one at a time: the
+// block's warps cover one another's gathers (300 nets of 20000 pins: 4973 us; four
+// pins in flight a thread, 6963 us).
 __device__ __forceinline__ Extent strided_extent(const float2 *xy, const int32_t *pin_cell,
                                                  const float *dx, const float *dy, long long b,
                                                  long long e, int t, int nt, int32_t C, bool &bad) {
   Extent q;
-  for (long long k0 = b + t; k0 < e; k0 += (long long)kPins * nt) {
-    float2 p[kPins];
-    pin_pos(xy, pin_cell, dx, dy, k0, nt, e, C, bad, p);
-#pragma unroll
-    for (int u = 0; u < kPins; ++u)
-      if (k0 + (long long)u * nt < e) q.add(p[u]);
+  for (long long k = b + t; k < e; k += nt) {
+    float2 p;
+    pin_pos<1>(xy, pin_cell, dx, dy, k, nt, e, C, bad, &p);
+    q.add(p);
   }
   return q;
 }
@@ -114,11 +115,16 @@ __device__ __forceinline__ Extent strided_extent(const float2 *xy, const int32_t
 // Bound by the latency of net_ptr -> pin_cell -> xy gathers: the next batch's
 // net_ptr is loaded a batch ahead, and a window's cell indices, then its gathers,
 // go out together (nothing is counted or branched on in between: the check of
-// an index used to end each gather's wait before the next index was loaded).  Windows take any batch (before, a batch
-// above its stage of 512 pins fell back to a lane per net straight from memory,
-// and every block looked through its nets once more for the long ones).  2.25M
-// nets, 8.9M pins: 150 -> 77 us (five blocks a SM spill: 96 us; eight pins in
-// flight a lane: 92 us).
+// an index used to end each gather's wait before the next index was loaded).
+// Windows take any batch (before, a batch above its stage of 512 pins fell back to
+// a lane per net straight from memory, and every block looked through its nets
+// once more for the long ones).  2.25M nets, 8.9M pins: 150 -> 77 us (five blocks
+// a SM spill: 96 us; eight pins in flight a lane: 92 us).
+// Long nets: spanned by the block whatever their number (those that did not fit a
+// list of eight used to be left to one warp, window by window: 20 nets of 500000
+// pins 71.9 ms, now 9.3 ms).  The pins are read by plain loads, so that a netlist
+// that L2 holds stays there for the next score (600k cells: 33.5 us with loads
+// that are evicted first, 27.9 us).
 __global__ void __launch_bounds__(kHpwlThreads, kHpwlPerSm) k_hpwl(const int64_t *net_ptr,
                                                           const int32_t *pin_cell,
                                                           const float *dx, const float *dy,
@@ -127,13 +133,13 @@ __global__ void __launch_bounds__(kHpwlThreads, kHpwlPerSm) k_hpwl(const int64_t
   __shared__ double red[kHpwlThreads / 32];
   __shared__ int last;
   __shared__ float2 stage_all[kHpwlThreads / 32][kHpwlWin];
-  __shared__ int32_t bigs[kHpwlThreads / 32][kHpwlBigs];
-  __shared__ int nbigs[kHpwlThreads / 32];
+  __shared__ int32_t list[kHpwlThreads / 32][kHpwlList + 1];
+  __shared__ int nlongs[kHpwlThreads / 32];
   __shared__ float4 mm[kHpwlThreads / 32];
   float2 *stg = stage_all[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   dfl acc{0.f, 0.f};
-  int nbig = 0;  // the same in every lane
+  int nlong = 0;  // the same in every lane
   bool bad = false;
   const long long wg = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long step = (((long long)gridDim.x * blockDim.x) >> 5) * 32;
@@ -150,31 +156,33 @@ __global__ void __launch_bounds__(kHpwlThreads, kHpwlPerSm) k_hpwl(const int64_t
       nz = ptr(base + step + lane + 1);
     }
     const long long p0 = __shfl_sync(0xffffffffu, a, 0), p1 = __shfl_sync(0xffffffffu, z, 31);
-    bool big = z - a > kHpwlWarpMax;
-    unsigned bb = __ballot_sync(0xffffffffu, big);
-    for (unsigned t = bb; t; t &= t - 1) {  // kept for the block while the list has room
+    const bool isl = z - a > kHpwlWarpMax;
+    for (unsigned t = __ballot_sync(0xffffffffu, isl); t; t &= t - 1) {  // kept for later
       const int src = __ffs(t) - 1;
-      if (nbig < kHpwlBigs) {
-        if (lane == 0) bigs[wid][nbig] = (int32_t)(base + src);
-        ++nbig;
-      } else {
-        if (lane == src) big = false;  // spanned below, window by window
-        bb &= ~(1u << src);
+      if (nlong < kHpwlList) {
+        if (lane == 0) list[wid][nlong] = (int32_t)(base + src);
+      } else if (nlong == kHpwlList && lane == 0) {
+        list[wid][kHpwlList] = (int32_t)(base + src);  // the first that the list does not hold
       }
+      nlong = min(nlong + 1, kHpwlList + 1);
     }
     Extent q;
     for (long long c0 = p0; c0 < p1;) {
-      if (bb) {  // a window starts behind a net that is left out
-        const unsigned in = __ballot_sync(0xffffffffu, big && a <= c0 && c0 < z);
-        if (in) {
-          c0 = __shfl_sync(0xffffffffu, z, __ffs(in) - 1);
+      // a window ends at the next long net and starts behind one
+      long long e1 = p1;
+      const unsigned nx = __ballot_sync(0xffffffffu, isl && z > c0);
+      if (nx) {
+        const long long la = __shfl_sync(0xffffffffu, a, __ffs(nx) - 1);
+        if (la <= c0) {
+          c0 = __shfl_sync(0xffffffffu, z, __ffs(nx) - 1);
           continue;
         }
+        e1 = la;
       }
-      const int n = (int)(p1 - c0 < kHpwlWin ? p1 - c0 : kHpwlWin);
+      const int n = (int)(e1 - c0 < kHpwlWin ? e1 - c0 : kHpwlWin);
       for (int k0 = 0; k0 < n; k0 += kPins * 32) {
         float2 p[kPins];
-        pin_pos(xy, pin_cell, dx, dy, c0 + k0 + lane, 32, c0 + n, C, bad, p);
+        pin_pos<kPins>(xy, pin_cell, dx, dy, c0 + k0 + lane, 32, c0 + n, C, bad, p);
 #pragma unroll
         for (int u = 0; u < kPins; ++u)
           if (k0 + 32 * u + lane < n) stg[k0 + 32 * u + lane] = p[u];
@@ -182,8 +190,7 @@ __global__ void __launch_bounds__(kHpwlThreads, kHpwlPerSm) k_hpwl(const int64_t
       __syncwarp();
       // this lane's net's part of the window
       const int lo = (int)(a > c0 ? (a - c0 < n ? a - c0 : n) : 0);
-      int hi = (int)(z > c0 ? (z - c0 < n ? z - c0 : n) : 0);
-      if (big) hi = lo;
+      const int hi = (int)(z > c0 ? (z - c0 < n ? z - c0 : n) : 0);
       const bool wide = hi - lo > kHpwlLane;
       if (!wide)
         for (int k = lo; k < hi; ++k) q.add(stg[k]);
@@ -198,20 +205,34 @@ __global__ void __launch_bounds__(kHpwlThreads, kHpwlPerSm) k_hpwl(const int64_t
       __syncwarp();
       c0 += n;
     }
-    if (!big && z > a) {
+    if (!isl && z > a) {
       q.close();
       span_add(acc, q.x0, q.x1, q.y0, q.y1);
     }
   }
-  // the block's nets of more than kHpwlWarpMax pins, warp by warp, in order
-  if (lane == 0) nbigs[wid] = nbig;
+  // The block's long nets, warp by warp, in order.  Those that a warp's list does not
+  // hold are found by looking through its batches from there once more.
+  if (lane == 0) nlongs[wid] = nlong;
+  auto long_nets = [&](int w, auto f) {  // the same in every thread
+    for (int i = 0; i < min(nlongs[w], kHpwlList); ++i) {
+      const long long e = list[w][i];
+      f(net_ptr[e], net_ptr[e + 1]);
+    }
+    if (nlongs[w] <= kHpwlList) return;
+    const long long first = list[w][kHpwlList];
+    for (long long base = first & ~31LL; base < M; base += step) {
+      const long long e = base + lane, a = ptr(e), z = ptr(e + 1);
+      for (unsigned t = __ballot_sync(0xffffffffu, z - a > kHpwlWarpMax && e >= first); t; t &= t - 1) {
+        const int src = __ffs(t) - 1;
+        f(__shfl_sync(0xffffffffu, a, src), __shfl_sync(0xffffffffu, z, src));
+      }
+    }
+  };
   __syncthreads();
   double bigacc = 0.0;  // thread 0
   for (int w = 0; w < kHpwlThreads / 32; ++w)
-    for (int i = 0; i < nbigs[w]; ++i) {
-      const long long e = bigs[w][i];
-      Extent r = strided_extent(xy, pin_cell, dx, dy, net_ptr[e], net_ptr[e + 1], threadIdx.x,
-                                kHpwlThreads, C, bad);
+    long_nets(w, [&](long long a, long long z) {
+      Extent r = strided_extent(xy, pin_cell, dx, dy, a, z, threadIdx.x, kHpwlThreads, C, bad);
       r.warp();
       if (lane == 0) mm[wid] = make_float4(r.x0, r.x1, r.y0, r.y1);
       __syncthreads();
@@ -225,7 +246,7 @@ __global__ void __launch_bounds__(kHpwlThreads, kHpwlPerSm) k_hpwl(const int64_t
         bigacc += ((double)r.x1 - (double)r.x0) + ((double)r.y1 - (double)r.y0);
       }
       __syncthreads();
-    }
+    });
   if (bad) atomicAdd(ticket + 1, 1);
   const double accd = warp_sum(df_to_d(df_norm(acc)));
   if (lane == 0) red[wid] = accd;
