@@ -1,6 +1,7 @@
 """pl_hpwl with more long nets than a warp's list holds, in one batch and over
 several of the warp's batches, against the oracle (1e-5 relative, the bar of the
-other HPWL tests); and the time of long nets, which is that of their number."""
+other HPWL tests); the time of long nets, which is that of their number, and of
+nets just above what a lane spans alone."""
 import time
 
 import numpy as np
@@ -61,3 +62,7 @@ def _time(sizes):
 
 def test_time_of_long_nets_is_linear():
     assert _time([200000] * 24) <= 1.25 * 3 * _time([200000] * 8)
+
+
+def test_nets_of_17_pins_take_little_longer_than_of_16():
+    assert _time([17] * 400000) <= 1.25 * _time([16] * 400000)
