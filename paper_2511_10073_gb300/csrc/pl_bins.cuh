@@ -97,8 +97,9 @@ __device__ __forceinline__ void bin_slot_group(const void *bwq, size_t wbase, co
   }
 }
 
-// Chunk c's partials (a warp).  NINE: the window is known to have 9 slots.
-template <int WT, bool DEG, bool NINE>
+// Chunk c's partials (a warp).  NINE: the window is known to have 9 slots; FIVE:
+// they are taken as groups of five and four.
+template <int WT, bool DEG, bool NINE, bool FIVE = false>
 __device__ __forceinline__ void bin_chunk(const BinGeo &B, const int32_t *bchunk,
                                           const int32_t *cown, const int64_t *boff,
                                           const uint32_t *blist, const void *bwq,
@@ -123,8 +124,16 @@ __device__ __forceinline__ void bin_chunk(const BinGeo &B, const int32_t *bchunk
   const int nu = (int)((min(k1 - k0, (long long)kBinChunk) + 31) / 32);
   const size_t pb = (size_t)c * B.W;
   if (NINE) {  // the 3 x 3 window of 20 to 39 bins: mostly full chunks
-    // (three groups of three in a rolled loop hold in 64 registers; groups of
-    // five and four, unrolled, spilled)
+    // (three groups of three in a rolled loop; groups of five and four spill when
+    // unrolled, and hold in 64 registers only alone in their kernel and rolled)
+    if (FIVE) {
+#pragma unroll 1
+      for (int t0 = 0; t0 < 9; t0 += 5) {
+        if (t0 == 0) bin_slot_group<WT, DEG, 5, false>(bwq, wbase, cv, nu, xi, part, pb, 0);
+        else bin_slot_group<WT, DEG, 4, false>(bwq, wbase, cv, nu, xi, part, pb, 5);
+      }
+      return;
+    }
 #pragma unroll 1
     for (int t0 = 0; t0 < 9; t0 += 3)
       bin_slot_group<WT, DEG, 3, false>(bwq, wbase, cv, nu, xi, part, pb, t0);
@@ -156,7 +165,10 @@ __global__ void __launch_bounds__(kBinThreads, 8) k_bin_partials(BinGeo B, const
   const int nchunk = bchunk[B.NB];
   for (long long c = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; c < nchunk;
        c += ((long long)gridDim.x * blockDim.x) >> 5)
-    bin_chunk<WT, DEG, NINE>(B, bchunk, cown, boff, blist, bwq, x, part, c);
+    // FP32 weights: more of the longer loads in flight beside the short rows (filter
+    // of 2.2M cells, eight powers: 1471 us by threes, 1454 us by five and four;
+    // BF16: 1401 and 1424 us)
+    bin_chunk<WT, DEG, NINE, WT == 0 && !DEG>(B, bchunk, cown, boff, blist, bwq, x, part, c);
 }
 
 template <bool DEG>
