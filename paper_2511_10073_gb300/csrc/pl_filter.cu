@@ -45,6 +45,7 @@ struct StepArgs {
   const void *hw;
   // work units of the applied matrix
   int64_t nrows;  // rows of the applied matrix
+  int32_t runs;   // the cells' rows as one run per block
   const int32_t *lrow;
   const uint64_t *lsb, *lhb;
   const uint32_t *lsl, *lhl;
@@ -527,15 +528,21 @@ template <int WT, int MODE>
 __global__ void __launch_bounds__(kRowThreads, 6) k_spmm_rows(StepArgs A) {
   constexpr int RPW = 32 / kRowLanes, WPB = kRowThreads / 32;
   const int wid = threadIdx.x >> 5;
-  // cells: a run of consecutive row groups per block, so that the neighbours'
+  // Cells: a run of consecutive row groups per block, so that the neighbours'
   // coordinates (mostly within a few thousand cells) stay in the SM's L1 (a round
-  // of 2.2M cells: 2239 us with the groups dealt to the blocks in turn, 2195 us)
-  const long long nc = A.C / RPW, per = (nc + gridDim.x - 1) / gridDim.x;
-  const long long c0 = blockIdx.x * per, c1 = c0 + per < nc ? c0 + per : nc;
-  for (long long k = c0 + wid; k < c1; k += WPB) rows_group<WT, MODE>(A, k * RPW);
-  // the other rows (macro pins, stars: very uneven) dealt in turn
-  const long long gw = (long long)blockIdx.x * WPB + wid, nw = (long long)gridDim.x * WPB;
-  for (long long base = (nc + gw) * RPW; base < A.nrows; base += nw * RPW) rows_group<WT, MODE>(A, base);
+  // of 2.2M cells: 2239 us with the groups dealt to the blocks in turn, 2195 us).
+  // Dealt in turn where the runs are unevenly long in entries (cells numbered by
+  // their number of nets, whose longest rows would be a few blocks' runs: eight
+  // powers of 2.2M such cells 1537 us as runs, 1431 us dealt), and below 16 passes
+  // of the grid, which the runs' ends do not fill (GiFt of 5k cells 85 us as runs,
+  // 72 us dealt; eight powers of 320k cells on 16 x 16 bins 296 and 281 us, of 1M
+  // cells 682 and 668 us, of 2M cells 1283 and 1320 us).
+  const int n = (int)((A.nrows + RPW - 1) / RPW), nw = gridDim.x * WPB;
+  const int nc = A.runs && n >= 16 * nw ? A.C / RPW : 0, per = (nc + gridDim.x - 1) / gridDim.x;
+  const int c0 = blockIdx.x * per, c1 = min(c0 + per, nc);
+  for (int k = c0 + wid; k < c1; k += WPB) rows_group<WT, MODE>(A, (long long)k * RPW);
+  // the other rows (macro pins, stars: very uneven) always in turn
+  for (int k = nc + blockIdx.x * WPB + wid; k < n; k += nw) rows_group<WT, MODE>(A, (long long)k * RPW);
 }
 
 // A GiFt chain pair over the short rows of the static matrix: the same
@@ -926,7 +933,7 @@ static cudaError_t launch_step(const StepArgs &A, double bytes, int wdtype, cuda
       return e != cudaSuccess ? e : cudaGetLastError();
     }
   }
-  // short rows: one wave of resident blocks, row groups dealt round robin
+  // short rows: one wave of resident blocks
   int *occ = g->occ_rows[MODE];
   const int wi = wdtype == PL_W_BF16 ? 1 : 0;
   if (!occ[wi]) {
@@ -1130,6 +1137,7 @@ pl_status run_gift(pl_graph *g, const pl_params *p, const float *in, float *out,
   StepArgs A{};
   fill_matrix(A, g->st, nullptr);
   A.C = g->C;
+  A.runs = g->even_rows;
   const double bytes = spmm_bytes((double)(g->st.nnz_s + g->st.nnz_l), (double)N, g->wdtype);
   fill_nodes(A, g);
   A.acc = P<double2>(g->acc);
@@ -1260,6 +1268,7 @@ static void hr_args(pl_graph *g, StepArgs &A) {
   A.hbwq = g->hbwq.p;
   A.hbin = P<int32_t>(g->hbin);
   A.C = g->C;
+  A.runs = g->even_rows;
   A.bn0 = g->Nst + g->Mm;
   A.B.nbx = g->nbx;
   A.B.nby = g->nby;

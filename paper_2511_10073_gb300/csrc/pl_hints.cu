@@ -548,10 +548,11 @@ struct LayIn {
   int may;  // static matrix: rows longer than this may become hub rows of the hint matrix
 };
 // Totals of a layout (device and host); may_*: static rows beyond LayIn::may
-// that are no hub rows, and their entries.
+// that are no hub rows, and their entries; cell_*: short entries of the static
+// matrix' blocks of cells' rows, in all and the most of one block.
 struct LayTotals {
-  unsigned long long s, l, may_entries;
-  uint32_t f, c, may_rows, pad;
+  unsigned long long s, l, may_entries, cell_sum;
+  uint32_t f, c, may_rows, cell_max;
 };
 
 // Lengths of row v of a split matrix.  Static matrix: hub when longer than
@@ -665,6 +666,10 @@ __global__ void __launch_bounds__(256) k_lay_sum(LayIn A, LaySum *bsum, LayTotal
     a.c += w[k].c;
   }
   bsum[blockIdx.x] = a;
+  if (!HINT && (blockIdx.x + 1LL) * kLayRows <= A.G.C) {
+    atomicAdd(&tot->cell_sum, a.s);
+    atomicMax(&tot->cell_max, (uint32_t)a.s);
+  }
 }
 
 // Exclusive scan of the block sums in place, totals to tot (one block).
@@ -1597,6 +1602,7 @@ pl_status prepare_static_layout(pl_graph *g, const int32_t *cnt, cudaStream_t s)
   LayIn A{};
   A.G.N = N;
   A.G.Nst = g->Nst;
+  A.G.C = g->C;
   A.cnt = cnt;
   A.may = kLong - g->W - kMacroSlots;
   LaySum *bsum;
@@ -1618,6 +1624,7 @@ pl_status prepare_static_layout(pl_graph *g, const int32_t *cnt, cudaStream_t s)
   lay_totals(m, t);
   g->may_rows = t.may_rows;
   g->may_entries = t.may_entries;
+  g->even_rows = 2.0 * (double)t.cell_max * (g->C / kLayRows) <= 3.0 * (double)t.cell_sum;
   TRY(lay_hub_arrays(m, t.f, t.c));
   if (t.f) {
     k_lay_apply<false, false, true><<<nblk, 256, 0, s>>>(A, lay_out(g, m), bsum, tot);

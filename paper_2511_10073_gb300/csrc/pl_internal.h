@@ -109,6 +109,7 @@ struct pl_graph {
   pl::Buf Db, phi;     // double [NB]
   // short static rows that may become hub rows of a hint matrix, and their entries
   uint64_t may_rows = 0, may_entries = 0;
+  bool even_rows = true;  // no 2048 cells' short static rows hold above 1.5 times the mean
   pl::Buf mac_base;    // uint64 [C] entry offset of a cell's first macro entry
   // bin hints without stored columns: each hint cell's window block and the
   // bin rows as its transpose over the bucket lists
