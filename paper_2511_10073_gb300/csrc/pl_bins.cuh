@@ -243,8 +243,11 @@ __device__ __forceinline__ void bin_row_chunks(const BinGeo &B, int b, const int
 }
 
 // First chunk of each bin's hint bucket and the bucket of each chunk, by one
-// block (a thread per bin, 1024 at a time, writes its bucket's chunks).
+// block: a thread per bin, 1024 at a time, writes its bucket's chunks, those of a
+// bin with more than kBinChunksLane the whole warp (hint build of 2.2M cells in one
+// bin, 8600 chunks: 605 -> 592 us).
 constexpr int kBinsOneBlock = 16384;
+constexpr int kBinChunksLane = 64;
 static __global__ void __launch_bounds__(1024) k_bin_chunks(int NB, const int64_t *boff,
                                                             int32_t *bchunk, int32_t *cown) {
   __shared__ int ws[32];
@@ -273,7 +276,14 @@ static __global__ void __launch_bounds__(1024) k_bin_chunks(int NB, const int64_
     __syncthreads();
     const int c0 = carry + (w ? ws[w - 1] : 0) + x - n;
     if (b < NB) bchunk[b] = c0;
-    for (int c = 0; c < n; ++c) cown[c0 + c] = b;
+    const bool wide = n > kBinChunksLane;
+    if (!wide)
+      for (int c = 0; c < n; ++c) cown[c0 + c] = b;
+    for (unsigned t = __ballot_sync(0xffffffffu, wide); t; t &= t - 1) {
+      const int src = __ffs(t) - 1;
+      const int m = __shfl_sync(0xffffffffu, n, src), at = __shfl_sync(0xffffffffu, c0, src);
+      for (int c = lane; c < m; c += 32) cown[at + c] = b - lane + src;
+    }
     carry += ws[31];
     __syncthreads();
   }
