@@ -193,22 +193,6 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
-// Ascending bitonic sort of one key per lane across a warp.
-template <typename K>
-__device__ __forceinline__ K warp_bitonic(K key, int lane) {
-#pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      K other = __shfl_xor_sync(0xffffffffu, key, j);
-      bool up = (lane & k) == 0;
-      bool lower = (lane & j) == 0;
-      key = (lower == up) ? (other < key ? other : key) : (other > key ? other : key);
-    }
-  }
-  return key;
-}
-
 // Ascending bitonic sort of n (power of two) keys in shared memory by a CTA.
 template <typename K>
 __device__ void cta_bitonic(K *a, int n) {
@@ -237,53 +221,6 @@ __device__ __forceinline__ long long co_rank(const K *A, long long na, const K *
     if (A[mid] <= B[d - mid - 1]) lo = mid + 1; else hi = mid;
   }
   return lo;
-}
-
-// CTA-cooperative stable merge of sorted A and B into C (all global).
-template <typename K>
-__device__ void cta_merge(const K *A, long long na, const K *B, long long nb, K *C) {
-  const long long n = na + nb;
-  const int E = 16;
-  for (long long base = 0; base < n; base += (long long)blockDim.x * E) {
-    long long d0 = base + (long long)threadIdx.x * E;
-    if (d0 >= n) continue;
-    long long d1 = d0 + E < n ? d0 + E : n;
-    long long i = co_rank(A, na, B, nb, d0);
-    long long j = d0 - i;
-    for (long long d = d0; d < d1; ++d) {
-      bool takeA = j >= nb || (i < na && A[i] <= B[j]);
-      C[d] = takeA ? A[i++] : B[j++];
-    }
-  }
-}
-
-// Merge adjacent sorted runs of `src` pairwise until one run is left.
-// run_off[0..nruns] are run boundaries relative to src (modified).  Uses
-// `tmp` (same length) as ping-pong space; the result ends in src.
-template <typename K>
-__device__ void cta_merge_runs(K *src, K *tmp, long long *run_off, int nruns) {
-  K *a = src, *b = tmp;
-  while (nruns > 1) {
-    for (int r = 0; r + 1 < nruns; r += 2)
-      cta_merge(a + run_off[r], run_off[r + 1] - run_off[r], a + run_off[r + 1],
-                run_off[r + 2] - run_off[r + 1], b + run_off[r]);
-    if (nruns & 1)
-      for (long long q = run_off[nruns - 1] + threadIdx.x; q < run_off[nruns]; q += blockDim.x)
-        b[q] = a[q];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int w = 0;
-      for (int r = 0; r < nruns; r += 2) run_off[w++] = run_off[r];
-      run_off[w] = run_off[nruns];
-    }
-    __syncthreads();
-    nruns = (nruns + 1) >> 1;
-    K *t = a; a = b; b = t;
-  }
-  if (a != src) {
-    for (long long q = run_off[0] + threadIdx.x; q < run_off[1]; q += blockDim.x) src[q] = a[q];
-    __syncthreads();
-  }
 }
 
 // ------------------------------------------------------- host utilities
@@ -353,13 +290,12 @@ cudaError_t exclusive_scan(const Tin *in, Tout *out, long long n, void *tmp, cud
 //   MODE_SORT   : sort only (keys unique or order of equal keys irrelevant)
 //   MODE_UNIQUE : sort, then move the distinct keys to the segment start and
 //                 write their count to cnt[s]
-//   MODE_MERGE  : keys are (col << 32 | uint32 value) (64-bit keys) or
-//                 (col << 4 | code) (32-bit keys, values decoded by the merge
-//                 context below); sort, then for each distinct col write
+//   MODE_MERGE  : keys are (col << 4 | code), values decoded by the merge
+//                 context below; sort, then for each distinct col write
 //                 (col, sum of values as int64; a negative value is kept as
 //                 is) to mcol/mval at the segment start and the count to cnt[s]
 enum { MODE_SORT = 0, MODE_UNIQUE = 1, MODE_MERGE = 2 };
-// Value of a 32-bit merge key's code in segment (row) s: code c >= 1 is a
+// Value of a merge key's code in segment (row) s: code c >= 1 is a
 // clique pair of weight 1/c in lattice units (lattice / c); code 0 is a star
 // edge, value -p for the star's net of p nodes, the star node being the row
 // when the row is one, else the column.

@@ -788,12 +788,6 @@ __global__ void k_grid_geo(long long n, const uint32_t *list, const int32_t *mac
   }
 }
 
-__global__ void k_i32_to_i64(const int32_t *a, int64_t *b, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    b[i] = a[i];
-}
-
 __global__ void k_i64_to_i32(const int64_t *a, int32_t *b, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)

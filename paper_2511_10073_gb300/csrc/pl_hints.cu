@@ -59,14 +59,6 @@ __device__ __forceinline__ bool overlaps(float x, float y, float w, float h, flo
 }
 __device__ __forceinline__ int grid_of(float x, float x0, float sc, int n) { return bin_of(x, x0, sc, n); }
 
-// e^{-r} for r >= 0 carried in FP64: FP32 exp of the rounded argument times
-// the first-order correction for the rounding residue.
-__device__ __forceinline__ float exp_neg(double r) {
-  float rh = __double2float_rn(r);
-  float rl = __double2float_rn(r - (double)rh);
-  return expf(-rh) * (1.0f - rl);
-}
-
 // BF16 storage rounds the FP64 weight of the definition once.  The fast FP32
 // value is within a few FP32 ulps of it (FP32 exp: 2 ulps, three roundings),
 // so it rounds to the same bf16 unless it lies within kNearTie FP32 ulps of a
@@ -96,21 +88,6 @@ __device__ __noinline__ double macro_w_exact(float x, float y, float xm, float y
   return -__dmul_rn(exp_cw(-r), bw);
 }
 
-// Writes the stored form of v and returns the value it stores.
-__device__ __forceinline__ float store_w(void *wbuf, int wdtype, uint64_t k, float v) {
-  if (wdtype == PL_W_BF16) {
-    uint16_t h = f2bf16(v);
-    reinterpret_cast<uint16_t *>(wbuf)[k] = h;
-    return bf16_to_f(h);
-  }
-  reinterpret_cast<float *>(wbuf)[k] = v;
-  return v;
-}
-// BF16 store of an exactly rounded FP64 weight.
-__device__ __forceinline__ float store_bits(void *wbuf, uint64_t k, uint16_t h) {
-  reinterpret_cast<uint16_t *>(wbuf)[k] = h;
-  return bf16_to_f(h);
-}
 __device__ __forceinline__ float load_w(const void *wbuf, int wdtype, uint64_t k) {
   if (wdtype == PL_W_BF16) return bf16_to_f(reinterpret_cast<const uint16_t *>(wbuf)[k]);
   return reinterpret_cast<const float *>(wbuf)[k];
@@ -121,25 +98,6 @@ __device__ __forceinline__ void copy_w(void *dst, const void *src, int wdtype, u
     reinterpret_cast<uint16_t *>(dst)[kd] = reinterpret_cast<const uint16_t *>(src)[ks];
   else
     reinterpret_cast<float *>(dst)[kd] = reinterpret_cast<const float *>(src)[ks];
-}
-
-// Stores the stored form of v at k and, when k2 is not ~0, at k2 (the
-// transposed entry of a symmetric pair); returns the value it stores.
-__device__ __forceinline__ float store_w2(void *wbuf, int wdtype, uint64_t k, uint64_t k2, float v) {
-  if (wdtype == PL_W_BF16) {
-    const uint16_t h = f2bf16(v);
-    reinterpret_cast<uint16_t *>(wbuf)[k] = h;
-    if (k2 != ~0ull) reinterpret_cast<uint16_t *>(wbuf)[k2] = h;
-    return bf16_to_f(h);
-  }
-  reinterpret_cast<float *>(wbuf)[k] = v;
-  if (k2 != ~0ull) reinterpret_cast<float *>(wbuf)[k2] = v;
-  return v;
-}
-__device__ __forceinline__ float store_bits2(void *wbuf, uint64_t k, uint64_t k2, uint16_t h) {
-  reinterpret_cast<uint16_t *>(wbuf)[k] = h;
-  if (k2 != ~0ull) reinterpret_cast<uint16_t *>(wbuf)[k2] = h;
-  return bf16_to_f(h);
 }
 
 // Cells are taken in tiles of 2^tsh consecutive ids (hint_tile_shift) by the stable counting
@@ -871,7 +829,8 @@ __device__ __forceinline__ dfl df_absdiff(float uh, float ul, float c) {
 __device__ __forceinline__ bool df_ge(dfl a, dfl b) {
   return a.hi > b.hi || (a.hi == b.hi && a.lo >= b.lo);
 }
-// e^{-r} for r = hi + lo >= 0, the form of exp_neg.
+// e^{-r} for r = hi + lo >= 0: FP32 exp of r.hi times the first-order correction for
+// r.lo.
 __device__ __forceinline__ float exp_neg_df(dfl r) { return expf(-r.hi) * (1.0f - r.lo); }
 
 // (x - o) * s for a float x, o = oh + ol and s = sh + sl (double-floats), to
@@ -1110,7 +1069,7 @@ __global__ void __launch_bounds__(256, bf ? 4 : 3) k_assemble_hints(
         }
       }
       // window slots, row-major over the full window
-      const int b = cb, bx = b % G.nbx, by = b / G.nbx, wx = 2 * G.hx + 1;
+      const int b = cb, bx = b % G.nbx, by = b / G.nbx;
       const dfl ux = df_offset_scale(p.x, G.xlh, G.xll, G.iwh, G.iwl);
       const dfl uy = df_offset_scale(p.y, G.ylh, G.yll, G.ihh, G.ihl);
       uint16_t *wb16 = sb ? reinterpret_cast<uint16_t *>(sblk) + lane * W
@@ -1231,7 +1190,6 @@ __global__ void __launch_bounds__(256, bf ? 4 : 3) k_assemble_hints(
           }
         }
       }
-      (void)wx;
       mac_base[v] = mb;
     }
     dsum[v] = df_norm(Dl);

@@ -230,8 +230,6 @@ cudaError_t exclusive_scan(const Tin *in, Tout *out, long long n, void *tmp, cud
 template cudaError_t exclusive_scan<int32_t, int32_t>(const int32_t *, int32_t *, long long, void *, cudaStream_t);
 template cudaError_t exclusive_scan<int32_t, int64_t>(const int32_t *, int64_t *, long long, void *, cudaStream_t);
 template cudaError_t exclusive_scan<int64_t, int64_t>(const int64_t *, int64_t *, long long, void *, cudaStream_t);
-template cudaError_t exclusive_scan<uint32_t, uint64_t>(const uint32_t *, uint64_t *, long long, void *, cudaStream_t);
-template cudaError_t exclusive_scan<uint64_t, uint64_t>(const uint64_t *, uint64_t *, long long, void *, cudaStream_t);
 template cudaError_t exclusive_scan<uint8_t, int32_t>(const uint8_t *, int32_t *, long long, void *, cudaStream_t);
 
 // --------------------------------------------------------- segmented sort
@@ -240,8 +238,7 @@ constexpr int SEG_CAP = 4096;  // keys sorted in shared memory at once
 
 template <typename K>
 __device__ __forceinline__ K key_max() { return ~K(0); }
-// Merge keys: (col << 32 | value) for 64-bit keys, (col << 4 | code) for
-// 32-bit keys with the value decoded from the merge context.
+// Merge keys: col << 4 | code, the value decoded from the merge context.
 __constant__ MergeCtx c_merge;
 static MergeCtx h_merge;  // source of the asynchronous copy (kept alive)
 
@@ -252,12 +249,10 @@ cudaError_t set_merge_ctx(const MergeCtx &c, cudaStream_t s) {
 
 template <typename K>
 __device__ __forceinline__ int32_t key_col(K k) {
-  if (sizeof(K) == 8) return (int32_t)((uint64_t)k >> 32);
   return (int32_t)((uint32_t)k >> 4);
 }
 template <typename K>
 __device__ __forceinline__ long long key_val(K k, long long s) {
-  if (sizeof(K) == 8) return (long long)(int32_t)(uint32_t)((uint64_t)k & 0xffffffffu);
   const uint32_t code = (uint32_t)k & 15u;
   if (code) return c_merge.latq[code];
   const long long col = (long long)((uint32_t)k >> 4);
@@ -817,7 +812,6 @@ cudaError_t segmented_sort(K *keys, const int64_t *off, long long nseg, long lon
 
 template cudaError_t segmented_sort<uint32_t, MODE_SORT>(uint32_t *, const int64_t *, long long, long long, int32_t *, int32_t *, int64_t *, void *, cudaStream_t, long long);
 template cudaError_t segmented_sort<uint32_t, MODE_UNIQUE>(uint32_t *, const int64_t *, long long, long long, int32_t *, int32_t *, int64_t *, void *, cudaStream_t, long long);
-template cudaError_t segmented_sort<uint64_t, MODE_MERGE>(uint64_t *, const int64_t *, long long, long long, int32_t *, int32_t *, int64_t *, void *, cudaStream_t, long long);
 template cudaError_t segmented_sort<uint32_t, MODE_MERGE>(uint32_t *, const int64_t *, long long, long long, int32_t *, int32_t *, int64_t *, void *, cudaStream_t, long long);
 
 }  // namespace pl
