@@ -29,8 +29,8 @@
  *   - Each pl_graph owns a second and a third stream.  Graph builds and the
  *     sparse products of larger designs fork part of their work onto them (an
  *     event recorded on the given stream)
- *     and join it back (the given stream waits on an event), so every call
- *     still completes in the order of the given stream.
+ *     and join it back (the given stream waits on an event), so every call,
+ *     also one that fails, still completes in the order of the given stream.
  *   - The library allocates no device memory.  A graph's device buffers are
  *     carved from a workspace the caller passes to pl_build_graph (sized by
  *     pl_workspace_size); pl_hpwl takes its own small workspace.  The
@@ -127,7 +127,8 @@ size_t pl_workspace_size(const pl_netlist *nl, const pl_params *p);
 /* A1 (+ A2/A3 when xy_nodes != NULL).  Builds the static instance graph of
  * `nl` (Sec. IV problem statement, Sec. V macro pin expansion) into *g:
  * creates the graph when *g == NULL, otherwise rebuilds it in place (the
- * netlist may differ).  ws: device memory of ws_bytes bytes, 256-byte aligned,
+ * netlist may differ; it first waits for what earlier calls queued on the
+ * graph's streams).  ws: device memory of ws_bytes bytes, 256-byte aligned,
  * owned by the caller, holding every device buffer of the graph; it needs no
  * initialisation, must stay allocated and untouched while the graph is in use,
  * and may be released after pl_graph_destroy or after a rebuild with another

@@ -732,11 +732,11 @@ __device__ __forceinline__ double f2d(float f) {
 
 // FP64 sum over blocks b of part[b][i] for weight i = kTH + 32 blockIdx.x + lane:
 // eight runs of consecutive blocks, a warp each (sixteen loads in flight), every
-// run in block order, then the runs in order.  Returned to warp 0.  A dependent
-// FP64 addition takes about 60 ns here, so one chain over a step's 128 blocks is
-// the whole cost: the sum and its Adam update took 16.2 us a step as a chain per
-// weight (and two launches), 13.4 us with the loads taken off the chain, 5.8
-// us as eight chains.
+// run in block order, then the runs in order.  Returned to warp 0.  Bound by the
+// chain of dependent FP64 additions: over a step's 128 blocks the sum and its Adam
+// update took 16.2 us as a chain per weight (and two launches), 13.4 us with the
+// loads taken off the chain, 5.8 us as eight chains.  (The sum's last FP64 bits
+// depend on the number of runs.)
 constexpr int kSegs = 8;
 __device__ __forceinline__ double sum_parts(const float *part, int nblk, double (*sh)[32]) {
   const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
