@@ -530,15 +530,16 @@ __global__ void __launch_bounds__(kRowThreads, 6) k_spmm_rows(StepArgs A) {
   const int wid = threadIdx.x >> 5;
   // Cells: a run of consecutive row groups per block, so that the neighbours'
   // coordinates (mostly within a few thousand cells) stay in the SM's L1 (a round
-  // of 2.2M cells: 2239 us with the groups dealt to the blocks in turn, 2195 us).
-  // Dealt in turn where the runs are unevenly long in entries (cells numbered by
-  // their number of nets, whose longest rows would be a few blocks' runs: eight
-  // powers of 2.2M such cells 1537 us as runs, 1431 us dealt), and below 16 passes
-  // of the grid, which the runs' ends do not fill (GiFt of 5k cells 85 us as runs,
-  // 72 us dealt; eight powers of 320k cells on 16 x 16 bins 296 and 281 us, of 1M
-  // cells 682 and 668 us, of 2M cells 1283 and 1320 us).
+  // of 2.2M cells: 2239 us with the groups dealt to the blocks in turn, 2195 us;
+  // its eight powers alone 1401 and 1376 us).  Dealt in turn with FP32 weights (1437
+  // us as runs, 1428 us dealt); where the runs are unevenly long in entries (cells
+  // numbered by their number of nets, whose longest rows would be a few blocks'
+  // runs: eight powers of 2.2M such cells 1518 and 1424 us); and below 16 passes of
+  // the grid, which the runs' ends do not fill (GiFt of 60k cells 108 and 104 us;
+  // eight powers of 320k cells on 16 x 16 bins 284 and 275 us, of 1M cells 680 and
+  // 662 us).
   const int n = (int)((A.nrows + RPW - 1) / RPW), nw = gridDim.x * WPB;
-  const int nc = A.runs && n >= 16 * nw ? A.C / RPW : 0, per = (nc + gridDim.x - 1) / gridDim.x;
+  const int nc = WT == 1 && A.runs && n >= 16 * nw ? A.C / RPW : 0, per = (nc + gridDim.x - 1) / gridDim.x;
   const int c0 = blockIdx.x * per, c1 = min(c0 + per, nc);
   for (int k = c0 + wid; k < c1; k += WPB) rows_group<WT, MODE>(A, (long long)k * RPW);
   // the other rows (macro pins, stars: very uneven) always in turn
