@@ -528,18 +528,23 @@ template <int WT, int MODE>
 __global__ void __launch_bounds__(kRowThreads, 6) k_spmm_rows(StepArgs A) {
   constexpr int RPW = 32 / kRowLanes, WPB = kRowThreads / 32;
   const int wid = threadIdx.x >> 5;
-  // Cells: a run of consecutive row groups per block, so that the neighbours'
-  // coordinates (mostly within a few thousand cells) stay in the SM's L1 (a round
-  // of 2.2M cells: 2239 us with the groups dealt to the blocks in turn, 2195 us;
-  // its eight powers alone 1401 and 1376 us).  Dealt in turn with FP32 weights (1437
-  // us as runs, 1428 us dealt); where the runs are unevenly long in entries (cells
-  // numbered by their number of nets, whose longest rows would be a few blocks'
-  // runs: eight powers of 2.2M such cells 1518 and 1424 us); and below 16 passes of
-  // the grid, which the runs' ends do not fill (GiFt of 60k cells 108 and 104 us;
-  // eight powers of 320k cells on 16 x 16 bins 284 and 275 us, of 1M cells 680 and
-  // 662 us).
+  // Row groups are dealt to the blocks in turn, or the cells' ones as one run of
+  // consecutive groups per block, which keeps the neighbours' coordinates (mostly
+  // within a few thousand cells) in the SM's L1 but ends less evenly.  Eight powers,
+  // us dealt and as runs.  Runs:
+  //  * BF16, 3 x 3 windows, from 14 passes of the grid: 1.3M cells 877 and 858, 2.2M
+  //    1446 and 1409 (GiFt 610 and 596); 1M 666 and 674, FP32 1.3M 933 and 931;
+  //  * where the last pass of dealing would be nearly empty: 450k cells, one-bin
+  //    windows 350 and 328, 3 x 3 390 and 383 (5.03 passes).
+  // Otherwise dealt: 400k cells, one-bin windows 303 and 320, 1.3M 753 and 803, 5 x 5
+  // windows 1476 and 1498; GiFt of 60k cells 104 and 108.  And always dealt where the
+  // runs would be uneven in entries: 2.2M cells numbered by their number of nets,
+  // whose longest rows are a few blocks' runs, 1424 and 1518.
   const int n = (int)((A.nrows + RPW - 1) / RPW), nw = gridDim.x * WPB;
-  const int nc = WT == 1 && A.runs && n >= 16 * nw ? A.C / RPW : 0, per = (nc + gridDim.x - 1) / gridDim.x;
+  const int W = MODE == MODE_GIFT ? 9 : A.B.W;
+  const bool run = A.runs && ((WT == 1 && W == 9 && n >= 14 * nw) ||
+                              (W <= 9 && n >= 4 * nw && n % nw < nw / 16));
+  const int nc = run ? A.C / RPW : 0, per = (nc + gridDim.x - 1) / gridDim.x;
   const int c0 = blockIdx.x * per, c1 = min(c0 + per, nc);
   for (int k = c0 + wid; k < c1; k += WPB) rows_group<WT, MODE>(A, (long long)k * RPW);
   // the other rows (macro pins, stars: very uneven) always in turn
