@@ -97,9 +97,9 @@ __device__ __forceinline__ void bin_slot_group(const void *bwq, size_t wbase, co
   }
 }
 
-// Chunk c's partials (a warp).  NINE: the window is known to have 9 slots; FIVE:
-// they are taken as groups of five and four.
-template <int WT, bool DEG, bool NINE, bool FIVE = false>
+// Chunk c's partials (a warp).  NS: the window is known to have 9 slots, or 1 (0:
+// any number); FIVE: nine are taken as groups of five and four.
+template <int WT, bool DEG, int NS, bool FIVE = false>
 __device__ __forceinline__ void bin_chunk(const BinGeo &B, const int32_t *bchunk,
                                           const int32_t *cown, const int64_t *boff,
                                           const uint32_t *blist, const void *bwq,
@@ -123,7 +123,11 @@ __device__ __forceinline__ void bin_chunk(const BinGeo &B, const int32_t *bchunk
   const size_t wbase = (size_t)c * B.W * kBinChunk;
   const int nu = (int)((min(k1 - k0, (long long)kBinChunk) + 31) / 32);
   const size_t pb = (size_t)c * B.W;
-  if (NINE) {  // the 3 x 3 window of 20 to 39 bins: mostly full chunks
+  if (NS == 1) {  // fewer than 20 bins
+    bin_slot_group<WT, DEG, 1, true>(bwq, wbase, cv, nu, xi, part, pb, 0);
+    return;
+  }
+  if (NS == 9) {  // the 3 x 3 window of 20 to 39 bins: mostly full chunks
     // (three groups of three in a rolled loop; groups of five and four spill when
     // unrolled, and hold in 64 registers only alone in their kernel and rolled)
     if (FIVE) {
@@ -155,7 +159,7 @@ __device__ __forceinline__ void bin_chunk(const BinGeo &B, const int32_t *bchunk
   }
 }
 
-template <int WT, bool DEG, bool NINE>
+template <int WT, bool DEG, int NS>
 __global__ void __launch_bounds__(kBinThreads, 8) k_bin_partials(BinGeo B, const int32_t *bchunk,
                                                               const int32_t *cown,
                                                               const int64_t *boff,
@@ -168,7 +172,7 @@ __global__ void __launch_bounds__(kBinThreads, 8) k_bin_partials(BinGeo B, const
     // FP32 weights: more of the longer loads in flight beside the short rows (filter
     // of 2.2M cells, eight powers: 1471 us by threes, 1454 us by five and four;
     // BF16: 1401 and 1424 us)
-    bin_chunk<WT, DEG, NINE, WT == 0 && !DEG>(B, bchunk, cown, boff, blist, bwq, x, part, c);
+    bin_chunk<WT, DEG, NS, WT == 0 && !DEG>(B, bchunk, cown, boff, blist, bwq, x, part, c);
 }
 
 template <bool DEG>
@@ -176,8 +180,11 @@ inline cudaError_t launch_bin_partials(int wt, int grid, cudaStream_t s, const B
                                        const int32_t *bchunk, const int32_t *cown,
                                        const int64_t *boff, const uint32_t *blist,
                                        const void *bwq, const float2 *x, float4 *part) {
-  auto k = wt == 2 ? (B.W == 9 ? k_bin_partials<1, DEG, true> : k_bin_partials<1, DEG, false>)
-                   : (B.W == 9 ? k_bin_partials<0, DEG, true> : k_bin_partials<0, DEG, false>);
+  // (one slot in a kernel of its own: 56 registers and no spills beside the short
+  // rows; eight powers of 320k cells on 16 x 16 bins, FP32, 271 -> 266 us)
+  const int ns = B.W == 9 || B.W == 1 ? B.W : 0;
+  auto k = wt == 2 ? (ns == 9 ? k_bin_partials<1, DEG, 9> : ns ? k_bin_partials<1, DEG, 1> : k_bin_partials<1, DEG, 0>)
+                   : (ns == 9 ? k_bin_partials<0, DEG, 9> : ns ? k_bin_partials<0, DEG, 1> : k_bin_partials<0, DEG, 0>);
   k<<<grid, kBinThreads, 0, s>>>(B, bchunk, cown, boff, blist, bwq, x, part);
   return cudaGetLastError();
 }

@@ -532,18 +532,23 @@ __global__ void __launch_bounds__(kRowThreads, 6) k_spmm_rows(StepArgs A) {
   // consecutive groups per block, which keeps the neighbours' coordinates (mostly
   // within a few thousand cells) in the SM's L1 but ends less evenly.  Eight powers,
   // us dealt and as runs.  Runs:
-  //  * BF16, 3 x 3 windows, from 14 passes of the grid: 1.3M cells 877 and 858, 2.2M
-  //    1446 and 1409 (GiFt 610 and 596); 1M 666 and 674, FP32 1.3M 933 and 931;
-  //  * where the last pass of dealing would be nearly empty: 450k cells, one-bin
-  //    windows 350 and 328, 3 x 3 390 and 383 (5.03 passes).
-  // Otherwise dealt: 400k cells, one-bin windows 303 and 320, 1.3M 753 and 803, 5 x 5
-  // windows 1476 and 1498; GiFt of 60k cells 104 and 108.  And always dealt where the
-  // runs would be uneven in entries: 2.2M cells numbered by their number of nets,
-  // whose longest rows are a few blocks' runs, 1424 and 1518.
-  const int n = (int)((A.nrows + RPW - 1) / RPW), nw = gridDim.x * WPB;
-  const int W = MODE == MODE_GIFT ? 9 : A.B.W;
-  const bool run = A.runs && ((WT == 1 && W == 9 && n >= 14 * nw) ||
-                              (W <= 9 && n >= 4 * nw && n % nw < nw / 16));
+  //  * BF16, 3 x 3 windows, from 4 passes of the grid (360k cells 346 and 340, 860k
+  //    595 and 590, 2.2M 1446 and 1409; 740k 526 and 535), below that not in the
+  //    middle of a pass (258k, 2.9 passes, 303 and 286; 300k, 3.4 passes, 318 and 327);
+  //  * FP32, and smaller windows, within 1/16 below and 1/8 above a whole number of
+  //    passes, where dealing ends with a nearly empty one: 450k cells (5.03 passes),
+  //    one-bin windows 350 and 328, 3 x 3 390 and 383;
+  //  * GiFt, from 4 passes: 740k cells, BF16 273 and 262, FP32 273 and 270.
+  // Otherwise dealt: 290k cells, one-bin windows (3.26) 258 and 286, 400k (4.5) 303
+  // and 320, 1.3M 753 and 803, 5 x 5 windows 1476 and 1498; GiFt of 60k cells 104 and
+  // 108.  And always dealt where the runs would be uneven in entries: 2.2M cells
+  // numbered by their number of nets, whose longest rows are a few blocks' runs,
+  // 1424 and 1518.
+  const int n = (int)((A.nrows + RPW - 1) / RPW), nw = gridDim.x * WPB, part = n % nw;
+  bool run = A.runs;
+  if (MODE == MODE_GIFT) run = run && n >= 4 * nw;
+  else if (WT == 1 && A.B.W == 9) run = run && (n >= 4 * nw || part < nw / 4 || part > nw / 4 * 3);
+  else run = run && A.B.W <= 9 && n >= 2 * nw && (part < nw / 8 || part > nw / 16 * 15);
   const int nc = run ? A.C / RPW : 0, per = (nc + gridDim.x - 1) / gridDim.x;
   const int c0 = blockIdx.x * per, c1 = min(c0 + per, nc);
   for (int k = c0 + wid; k < c1; k += WPB) rows_group<WT, MODE>(A, (long long)k * RPW);
@@ -697,7 +702,7 @@ __global__ void __launch_bounds__(kHubRows * 32) k_hub_rows(StepArgs A) {
 // completion before they touch memory.  A launch lets its own dependents in only
 // after that wait, so no more than one launch is ever ahead, and x is read with
 // coherent loads (it is written while a waiting launch already exists).
-template <int WT, bool NINE>
+template <int WT, int NS>
 __global__ void __launch_bounds__(256, 4) k_power_units(StepArgs A, long long nbin) {
   pdl_wait();
   pdl_release();
@@ -709,7 +714,7 @@ __global__ void __launch_bounds__(256, 4) k_power_units(StepArgs A, long long nb
   u -= A.nchunks;
   if (u < nbin) {
     if (u < A.bchunk[A.B.NB])
-      bin_chunk<WT, false, NINE>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, u);
+      bin_chunk<WT, false, NS>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, u);
     return;
   }
   u -= nbin;
@@ -927,8 +932,8 @@ static cudaError_t launch_step(const StepArgs &A, double bytes, int wdtype, cuda
       const bool prof = prof_on();
       if (prof) prof_begin(s, PROF_HR, bytes);
       const bool bf = wdtype == PL_W_BF16, nine = A.B.W == 9;
-      auto ku = bf ? (nine ? k_power_units<1, true> : k_power_units<1, false>)
-                   : (nine ? k_power_units<0, true> : k_power_units<0, false>);
+      auto ku = bf ? (nine ? k_power_units<1, 9> : k_power_units<1, 0>)
+                   : (nine ? k_power_units<0, 9> : k_power_units<0, 0>);
       cudaError_t e = launch_pdl(ku, (int)blocks, 256, 0, s, A, nbin);
       if (e == cudaSuccess)
         e = launch_pdl(bf ? k_power_hubs<1> : k_power_hubs<0>, (A.nlong + kHubRows - 1) / kHubRows,
@@ -1444,9 +1449,9 @@ __device__ __forceinline__ void batch_units(const StepArgs *As, const long long 
     } else {
       if (k < A.bchunk[A.B.NB]) {
         if (A.B.W == 9)
-          bin_chunk<WT, false, true>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, k);
+          bin_chunk<WT, false, 9>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, k);
         else
-          bin_chunk<WT, false, false>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, k);
+          bin_chunk<WT, false, 0>(A.B, A.bchunk, A.cown, A.boff, A.blist, A.hbwq, A.x, A.bpart, k);
       }
     }
   }
